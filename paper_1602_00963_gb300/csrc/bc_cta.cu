@@ -1,26 +1,32 @@
-// Per-source path for small graphs: every CTA runs whole sources on its own.
+// Per-source path, one source per CTA: every CTA runs whole sources on its own.
 //
 // The method is Brandes' (Alg. 1) with the level-synchronous forward sweep of Alg. 2 /
 // Alg. 3 and the successor-checking backward sweep of Alg. 4 / Alg. 5, one source at a
 // time.  On a graph of a few thousand vertices a level holds far too little work for the
-// whole GPU, and the grid-wide barriers of the per-source kernel dominate.  Here the loop
-// over sources of Alg. 1 is spread over the CTAs (the coarse-grained parallelism of
-// Sec. 3.3, applied to the SMs of one GPU): a CTA takes sources blockIdx.x, blockIdx.x +
-// gridDim.x, ..., runs each with CTA barriers only, and keeps the source's depth, sigma,
-// r and queue in shared memory when they fit (else in a per-CTA slice of global memory).
+// whole GPU, and on a road network a level is a ring of a few hundred vertices; grid-wide
+// barriers would dominate both.  Here the loop over sources of Alg. 1 is spread over the CTAs
+// (the coarse-grained parallelism of Sec. 3.3, applied to the SMs of one GPU): a CTA takes
+// sources blockIdx.x, blockIdx.x + gridDim.x, ... and runs each with CTA barriers only, one
+// barrier per level and sweep.
 //
-// Forward level l: a warp per frontier vertex v, lanes over its edges.  The
-// compare-and-swap that discovers w returns the previous depth, and sigma[w] += sigma[v]
-// (64-bit integer atomics, exact) whenever it was -1 or l, with a sticky overflow bit on a
-// carry or an overflowed parent.  When a level overflowed, each overflowed vertex of it
-// also gets its extended-range sigma (mantissa, exponent) summed over its parents.
-// Backward level d: sigma of w is taken as m 2^e (m in [0.5, 1)), r is stored scaled by
-// 2^e; a warp per vertex w of level d sums its successors' r, rescaled to w's exponent, in
-// float-float arithmetic (lanes in edge order, then a fixed-order warp reduction); then
-// delta = m * sum, r[w] = (1 + omega) / m + sum, and the CTA's BC partial of w grows by
-// (omega[s] + 1) * delta.  A second kernel sums the partials in CTA order.  Every sum has a
-// fixed order (a vertex's path depends on its degree only), so the result repeats bit for
-// bit from run to run.
+// What bounds it: dependent memory round trips of a level (a queue entry, its row, the states
+// of its neighbours) and L2 transactions.  So a vertex's state is one 16-byte record, read
+// with one load: its value (forward: sigma; backward: r, which replaces it), its level, its
+// exponent.  Small graphs keep value, level and queue in shared memory instead.
+//
+// Forward pass l handles the entries w of level l, once per arc: neighbours of level l - 1 are
+// parents, their sigma is summed (a pull in arc order: no sigma atomics, and the extended
+// range needs no pass of its own); neighbours not reached yet are claimed for level l + 1 by
+// an atomic maximum on their level and queued.  The levels carry the source's base, which
+// grows by the levels used, so records of earlier sources read as "not reached" and nothing is
+// reset between sources.  An entry of degree <= 4 notes which neighbours are its successors in
+// its queue entry, so the backward sweep loads those alone.
+// Backward level d: a vertex sums its successors' r in float-float arithmetic, delta = sigma *
+// sum, r = (1 + omega) / sigma + sum, and the CTA's BC partial grows by (omega[s] + 1) * delta.
+// When a sigma of the source passed 2^64 sigma is taken as m 2^e (m in [0.5, 1)) and r is kept
+// scaled by 2^e; other sources need no exponents.  A second kernel sums the partials in CTA
+// order.  Every sum has a fixed order (how a vertex is handled depends on its degree only), so
+// the result repeats bit for bit from run to run.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -34,23 +40,29 @@ namespace bcl {
 
 namespace {
 
-constexpr int kCtaThreads = 512;
-constexpr int kCtaWarps = kCtaThreads / 32;
-constexpr size_t kCtaSmemMax = 200 * 1024;  // per-CTA state kept in shared memory up to this
+constexpr int kRing = 2048;     // entries of a level kept in shared memory (state in global memory)
+constexpr int kThin = 4;        // degree up to which a row record holds the neighbours themselves
+constexpr int kGroupDeg = 32;   // above a lane's degree: eight lanes up to here, a warp beyond
+constexpr int kNarrowDeg = 8;   // graphs of at most this degree: lanes alone (no code for larger rows)
+constexpr uint32_t kBase0 = 2;  // first base: level base - 1 is never in use, nor 0
+constexpr uint32_t kBaseMax = 0x3f000000u;
+constexpr int kIdMask = 0xffffff;  // queue entries: vertex id (n <= 2^24), successor bits above
+constexpr size_t kCtaSmemMax = 224 * 1024;  // state kept in shared memory up to this
 
 struct CtaK {
   int n;
   const int32_t *__restrict__ rp;
   const int32_t *__restrict__ ci;
+  const int4 *__restrict__ row4;  // row records (k_cta_rows), or null: read rp and ci
   const int32_t *__restrict__ omega;
   const int32_t *__restrict__ src;
   int nsrc;
   int leaf_term;
+  int spread;         // a level's consecutive entries go to different warps (see cta_slot)
   double *bcp;        // [gridDim.x][n] per-CTA BC partials
-  char *gws;          // per-CTA global slices (state when not in shared memory, level offsets)
+  char *gws;          // per-CTA global slices
   size_t slice;       // bytes per slice
-  int in_smem;        // state arrays in shared memory
-  int clean;          // state in global memory already cleared (left clean by the last call)
+  int clean;          // slices hold a valid base and records (left so by the last call)
   unsigned long long *stats;  // reached pairs, their arcs, levels, deepest level (max),
                               // sources whose sigma passed 2^64
   const int32_t *tri;         // 2-degree triples (a, b, c), 3 ints each
@@ -64,358 +76,689 @@ struct CtaK {
   const int32_t *req;
 };
 
-// State of one source, n vertices: sigma u64 | r float2 | depth i32 | queue i32 | overflow
-// bits.  The global slice of a CTA holds this state when it is not in shared memory, then
-// the level offsets and the extended-range sigma (mantissa f64, exponent i32), touched
-// only for overflowed vertices.
-__host__ __device__ inline size_t cta_state_bytes(int n) {
-  return ((size_t)n * 24 + ((size_t)(n + 31) / 32) * 4 + 16 + 15) & ~(size_t)15;
-}
-__host__ __device__ inline size_t cta_extra_bytes(int n) {  // a multiple of 16: states follow
-  return (((size_t)(n + 2) * 4 + 15) / 16 * 16 + (size_t)n * 12 + 15) & ~(size_t)15;
-}
-
-// One source's state: per-vertex arrays plus the level offsets and extended-range sigma.
-struct CtaState {
-  unsigned long long *sig;
-  float2 *r;
-  int32_t *d;
-  int32_t *Q;
-  uint32_t *ovf;
-  int32_t *loff;
-  double *xm;
-  int32_t *xe;
+// One vertex of one source, state in global memory.  tag: (base + level) << 1, low bit set once
+// sigma passed 2^64; below base << 1: not reached by this source.  val: sigma modulo 2^64, or
+// the extended range's mantissa (with exponent e); after the vertex's backward step r (float2).
+struct __align__(16) Rec {
+  unsigned long long val;
+  uint32_t tag;
+  int32_t e;
 };
 
-// Carve a state: the per-vertex block at blk (cta_state_bytes), the rest at extra
-// (cta_extra_bytes).
-__device__ __forceinline__ CtaState cta_carve(char *blk, char *extra, int n) {
-  CtaState S;
-  S.sig = (unsigned long long *)blk;
-  S.r = (float2 *)(blk + (size_t)n * 8);
-  S.d = (int32_t *)(blk + (size_t)n * 16);
-  S.Q = S.d + n;
-  S.ovf = (uint32_t *)(S.Q + n);
-  S.loff = (int32_t *)extra;
-  S.xm = (double *)(extra + ((size_t)(n + 2) * 4 + 15) / 16 * 16);
-  S.xe = (int32_t *)(S.xm + n);
+__host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
+// Global slice of a CTA: bases | records | queue | level offsets (state in shared memory:
+// exponents | level offsets | queue); with triples a second state and c's records.
+__host__ __device__ inline size_t cta_state_bytes(int n, bool sm) {
+  return (sm ? al16((size_t)n * 4) + al16((size_t)n * 2) : (size_t)n * 16 + al16((size_t)n * 4)) +
+         al16(((size_t)n + 2) * 4);
+}
+// Shared-memory state, n < 32768 (levels and ids in 16 bits): val u64 | tag u16 (level << 1, low
+// bit: sigma passed 2^64, 0xffff: not reached) | reached bits | queue u16 (in the slice when it
+// does not fit).  Cleared per source.
+__host__ __device__ inline size_t cta_smem_bytes(int n, bool with_q) {
+  return al16((size_t)n * 8) + (with_q ? 2 : 1) * al16((size_t)n * 2) + al16(((size_t)n + 31) / 32 * 4);
+}
+__host__ __device__ inline bool cta_smem_q(int n) { return cta_smem_bytes(n, true) <= kCtaSmemMax; }
+constexpr uint32_t kSmFree = 0xffffu;
+
+template <bool SM>
+struct CtaState {  // state in global memory
+  Rec *rec;
+  int32_t *Q;
+  int32_t *loff;  // level offsets into Q
+  uint32_t base;
+};
+template <>
+struct CtaState<true> {  // state in shared memory
+  unsigned long long *val;
+  uint16_t *tag, *Q;
+  uint32_t *vis;
+  int32_t *e;     // global memory, valid for sources with overflow
+  int32_t *loff;  // global memory
+};
+
+template <bool SM>
+__device__ __forceinline__ CtaState<SM> cta_carve(char *smem, char *g, int n) {
+  CtaState<SM> S;
+  if constexpr (SM) {
+    S.val = (unsigned long long *)smem;
+    smem += al16((size_t)n * 8);
+    S.tag = (uint16_t *)smem;
+    smem += al16((size_t)n * 2);
+    S.vis = (uint32_t *)smem;
+    smem += al16(((size_t)n + 31) / 32 * 4);
+    S.e = (int32_t *)g;
+    S.loff = (int32_t *)(g + al16((size_t)n * 4));
+    S.Q = cta_smem_q(n) ? (uint16_t *)smem : (uint16_t *)(g + al16((size_t)n * 4) + al16(((size_t)n + 2) * 4));
+  } else {
+    S.rec = (Rec *)g;
+    S.Q = (int32_t *)(g + (size_t)n * 16);
+    S.loff = (int32_t *)(g + (size_t)n * 16 + al16((size_t)n * 4));
+    S.base = kBase0;
+  }
   return S;
 }
 
-constexpr int kCtaLaneDeg = 32;  // vertices of degree <= this are handled by one thread
-constexpr int kStage = 4;        // state in global memory: a thread's edges are loaded
-                                 // kStage at a time (their latencies overlap)
-constexpr int kStage2 = 2;       // the same for the 2-degree backward sweep
-constexpr int kCtaBig = 512;     // higher-degree vertices listed per pass for whole warps
+// Nothing reached: every tag free (shared memory), or below the first base.
+__device__ __forceinline__ void cta_clear(CtaState<true> &S, int n) {
+  for (int i = threadIdx.x; i < (int)(al16((size_t)n * 2) / 16); i += blockDim.x)
+    ((uint4 *)S.tag)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  for (int i = threadIdx.x; i < (n + 31) / 32; i += blockDim.x) S.vis[i] = 0u;
+}
+__device__ __forceinline__ void cta_clear(CtaState<false> &S, int n) {
+  for (int v = threadIdx.x; v < n; v += blockDim.x) S.rec[v].tag = 0u;
+  S.base = kBase0;
+}
 
 struct CtaShared {
-  int q, ovf, lovf[2], nbig;
+  int cnt[3];  // entries appended to level l (slot l % 3)
+  int ovf;
   unsigned long long ns;
-  int big[kCtaBig];
+  // statistics of the CTA's sources
+  unsigned long long arcs, reached, levels, deepest, ovf_sources;
 };
 
-// Entries Q[i0, i1): a vertex of degree <= kCtaLaneDeg is handled by one thread (a level of
-// a sparse, high-diameter graph then keeps every thread busy), a larger one by a whole warp
-// (lanes over its edges) from a shared list.  The entries are taken in windows of one per
-// thread, so the list (kCtaBig >= kCtaThreads) never fills: which path handles a vertex, and
-// so the order of its floating-point sums, depends on its degree only.
-static_assert(kCtaBig >= kCtaThreads, "a window's high-degree vertices must fit the list");
-template <typename LaneF, typename WarpF>
-__device__ __forceinline__ void cta_split(const CtaK &p, const int32_t *Q, int i0, int i1, CtaShared &sh,
-                                          LaneF &&lane_f, WarpF &&warp_f) {
-  for (int b = i0; b < i1; b += kCtaThreads) {  // uniform over the CTA
-    const int i = b + (int)threadIdx.x;
-    if (i < i1) {
-      const int v = Q[i];
-      if (p.rp[v + 1] - p.rp[v] > kCtaLaneDeg)
-        sh.big[atomicAdd(&sh.nbig, 1)] = v;
-      else
-        lane_f(v);
-    }
-    __syncthreads();
-    const int nb = sh.nbig;
-    __syncthreads();
-    if (threadIdx.x == 0) sh.nbig = 0;
-    for (int j = (int)(threadIdx.x >> 5); j < nb; j += kCtaWarps) warp_f(sh.big[j]);
-    __syncthreads();
+// row4[v] = the neighbours of v (-1 past the last) or, above kThin arcs, {-2, first arc, degree, 0}:
+// one 16-byte load instead of the row offsets and then the arcs.
+__global__ void k_cta_rows(int n, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int4 *row4) {
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+    const int a = rp[v], d = rp[v + 1] - a;
+    int4 q = make_int4(-2, a, d, 0);
+    if (d <= kThin)
+      q = make_int4(d > 0 ? ci[a] : -1, d > 1 ? ci[a + 1] : -1, d > 2 ? ci[a + 2] : -1, d > 3 ? ci[a + 3] : -1);
+    row4[v] = q;
   }
 }
 
-// sigma of v as m 2^e with m in [0.5, 1)
-__device__ __forceinline__ XS cta_sigma(const CtaState &S, int v) {
-  if ((S.ovf[v >> 5] >> (v & 31)) & 1u) {
+// A vertex's row: its degree, where its arcs start, and up to kThin neighbours (then e0 is unused).
+struct Row {
+  int deg, e0;
+  int4 nb;
+};
+template <bool SM>
+__device__ __forceinline__ Row cta_row(const CtaK &p, int v) {
+  Row r;
+  if (!SM && p.row4) {
+    r.nb = p.row4[v];
+    r.e0 = r.nb.y;
+    r.deg = r.nb.x == -2 ? r.nb.z : (r.nb.x >= 0) + (r.nb.y >= 0) + (r.nb.z >= 0) + (r.nb.w >= 0);
+  } else {
+    r.e0 = p.rp[v];
+    r.deg = p.rp[v + 1] - r.e0;
+    r.nb = make_int4(-1, -1, -1, -1);
+    if (!SM && r.deg <= kThin) {
+      if (r.deg > 0) r.nb.x = p.ci[r.e0];
+      if (r.deg > 1) r.nb.y = p.ci[r.e0 + 1];
+      if (r.deg > 2) r.nb.z = p.ci[r.e0 + 2];
+      if (r.deg > 3) r.nb.w = p.ci[r.e0 + 3];
+    }
+  }
+  return r;
+}
+__device__ __forceinline__ Row no_row() {
+  Row r;
+  r.deg = r.e0 = 0;
+  r.nb = make_int4(-1, -1, -1, -1);
+  return r;
+}
+// Arcs u .. u + 3 of a row (-1 past lim).
+template <bool SM>
+__device__ __forceinline__ void row_arcs(const CtaK &p, const Row &r, int u, int lim, int (&x)[4]) {
+  if (!SM && r.deg <= kThin) {
+    x[0] = r.nb.x;
+    x[1] = r.nb.y;
+    x[2] = r.nb.z;
+    x[3] = r.nb.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; j++) x[j] = u + j < lim ? p.ci[r.e0 + u + j] : -1;
+  }
+}
+
+// A record of the CTA's own slice, read while other threads of the CTA may raise its tag.
+__device__ __forceinline__ Rec ld_rec(const Rec *a) {
+  unsigned long long x, y;
+  asm volatile("ld.relaxed.cta.global.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(a) : "memory");
+  Rec r;
+  r.val = x;
+  r.tag = (uint32_t)y;
+  r.e = (int32_t)(y >> 32);
+  return r;
+}
+__device__ __forceinline__ void st_rec(Rec *a, const Rec &r) {
+  *(ulonglong2 *)a = make_ulonglong2(r.val, (unsigned long long)r.tag | ((unsigned long long)(uint32_t)r.e << 32));
+}
+
+// The record of x; from shared memory the value is read only where the tag is one of the
+// wanted level's (tag & ~1 == want), and the exponent only with ext.
+__device__ __forceinline__ Rec cta_rec(const CtaState<true> &S, int x, uint32_t want, bool ext) {
+  Rec r;
+  r.tag = *(volatile uint16_t *)&S.tag[x];
+  r.val = 0ull;
+  r.e = 0;
+  if ((r.tag & ~1u) == want) {
+    r.val = S.val[x];
+    if (ext) r.e = S.e[x];
+  }
+  return r;
+}
+__device__ __forceinline__ Rec cta_rec(const CtaState<false> &S, int x, uint32_t, bool) { return ld_rec(S.rec + x); }
+
+// sigma of a record as m 2^e with m in [0.5, 1)
+__device__ __forceinline__ XS rec_sigma(const Rec &r) {
+  if (r.tag & 1u) {
     XS x;
-    x.m = S.xm[v];
-    x.e = S.xe[v];
+    x.m = __longlong_as_double((long long)r.val);
+    x.e = r.e;
     return x;
   }
-  return xs_u64(S.sig[v]);
+  return xs_u64(r.val);
 }
-__device__ __forceinline__ int cta_exp(const CtaState &S, int v) {
-  return ((S.ovf[v >> 5] >> (v & 31)) & 1u) ? S.xe[v] : 64 - __clzll((long long)S.sig[v]);
+__device__ __forceinline__ float2 rec_r(const Rec &r) {
+  return make_float2(__uint_as_float((unsigned)r.val), __uint_as_float((unsigned)(r.val >> 32)));
+}
+__device__ __forceinline__ unsigned long long r_bits(float2 r) {
+  return (unsigned long long)__float_as_uint(r.x) | ((unsigned long long)__float_as_uint(r.y) << 32);
 }
 
-__device__ void cta_clear(const CtaState &S, int n) {
-  for (int v = threadIdx.x; v < n; v += kCtaThreads) {
-    S.sig[v] = 0ull;
-    S.d[v] = -1;
+// Which entry of a window of blockDim.x a thread takes: its own index, or (spread) consecutive
+// entries in different warps.  Graphs with rows beyond kThin spread, so that a few large rows
+// next to each other in the queue do not fall to one warp; others fill whole warps.
+__device__ __forceinline__ int cta_slot(const CtaK &p) {
+  const int tid = threadIdx.x;
+  return p.spread ? (tid & 31) * (int)(blockDim.x >> 5) + (tid >> 5) : tid;
+}
+
+// Rows beyond LD, one per lane of mask m, are taken 32 / W at a time by W lanes each.
+// group_take: the lane whose row this lane's group takes next (-1: none left); group_give: the
+// owners' copies of their group's value (rank: the owner's number among this batch's).
+template <int W>
+__device__ __forceinline__ int group_take(unsigned m) {
+  if constexpr (W == 32) {
+    return __ffs(m) - 1;
+  } else {
+    int mine = -1;
+#pragma unroll
+    for (int k = 0; k < 32 / W; k++) {
+      if (m && (int)lane_id() / W == k) mine = __ffs(m) - 1;
+      m &= m - 1;
+    }
+    return mine;
   }
-  for (int i = threadIdx.x; i < (n + 31) / 32; i += kCtaThreads) S.ovf[i] = 0u;
+}
+template <int W>
+__device__ __forceinline__ unsigned group_drop(unsigned m) {
+#pragma unroll
+  for (int k = 0; k < 32 / W; k++) m &= m - 1;
+  return m;
 }
 
-// Forward sweep from s (Alg. 2 / Alg. 3, CTA barriers).  Returns the deepest non-empty
-// level; *qtot = reached vertices, *arcs += their adjacency entries (lane 0 of each warp).
-__device__ int cta_forward(const CtaK &p, const CtaState &S, int s, CtaShared &sh, int *qtot,
-                           unsigned long long *arcs) {
-  const int tid = threadIdx.x, lane = tid & 31;
+// ------------------------------------------------------------------ forward
+// What a forward pass needs besides the graph and the state.
+struct FwdLevel {
+  uint32_t t0, tl;  // tags of level 0 and of this level (low bit clear)
+  int q1;           // queue position of the next level's first entry
+  int *cnt;         // its entries so far
+  int32_t *ring;    // state in global memory: its first kRing entries
+};
+template <bool SM>
+__device__ __forceinline__ bool unreached(const FwdLevel &f, uint32_t tag) {
+  return SM ? tag == kSmFree : tag < f.t0;
+}
+
+// Append the flagged lanes' vertices to the next level (one shared atomic per warp).
+__device__ __forceinline__ void fwd_put(const CtaState<true> &S, const FwdLevel &f, int pos, int x) {
+  S.Q[f.q1 + pos] = (uint16_t)x;
+}
+__device__ __forceinline__ void fwd_put(const CtaState<false> &S, const FwdLevel &f, int pos, int x) {
+  if (pos < kRing)
+    f.ring[pos] = x;
+  else
+    S.Q[f.q1 + pos] = x;
+}
+template <bool SM, int K>
+__device__ __forceinline__ void fwd_append(const CtaState<SM> &S, const FwdLevel &f, const bool (&nw)[K],
+                                           const int (&x)[K]) {
+  unsigned m[K];
+  int tot = 0;
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    m[k] = __ballot_sync(BC_FULL, nw[k]);
+    tot += __popc(m[k]);
+  }
+  if (!tot) return;
+  int base = 0;
+  if (lane_id() == 0) base = atomicAdd(f.cnt, tot);
+  base = __shfl_sync(BC_FULL, base, 0);
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    if (nw[k]) fwd_put(S, f, base + __popc(m[k] & lanemask_lt()), x[k]);
+    base += __popc(m[k]);
+  }
+}
+
+// Claim x for the next level; true for the one thread that does.
+__device__ __forceinline__ bool fwd_claim(const CtaState<true> &S, const FwdLevel &f, int x) {
+  const uint32_t bit = 1u << (x & 31);
+  if (atomicOr(&S.vis[x >> 5], bit) & bit) return false;
+  *(volatile uint16_t *)&S.tag[x] = (uint16_t)(f.tl + 2u);
+  return true;
+}
+__device__ __forceinline__ bool fwd_claim(const CtaState<false> &S, const FwdLevel &f, int x) {
+  return atomicMax(&S.rec[x].tag, f.tl + 2u) < f.t0;
+}
+
+// Store w's sigma: s modulo 2^64, or (ov: it passed 2^64) its extended range a.
+__device__ __forceinline__ void fwd_commit(const CtaState<true> &S, const FwdLevel &f, int w, unsigned long long s,
+                                           bool ov, bool xp, const XS &a) {
+  if (ov) {
+    S.tag[w] = (uint16_t)(f.tl | 1u);
+    if (!xp) {
+      s = (unsigned long long)__double_as_longlong(a.m);
+      S.e[w] = a.e;
+    }
+  }
+  S.val[w] = s;
+}
+__device__ __forceinline__ void fwd_commit(const CtaState<false> &S, const FwdLevel &f, int w, unsigned long long s,
+                                           bool ov, bool xp, const XS &a) {
+  if (!ov) {
+    S.rec[w].val = s;
+    return;
+  }
+  Rec r;
+  r.tag = f.tl | 1u;
+  r.val = xp ? s : (unsigned long long)__double_as_longlong(a.m);
+  r.e = a.e;
+  st_rec(S.rec + w, r);
+}
+
+__device__ __forceinline__ void sum_carry(unsigned long long &s, bool &ov, unsigned long long v, bool o) {
+  const unsigned long long t = s + v;
+  ov = ov || t < s || o;
+  s = t;
+}
+
+template <bool SM, int W>
+__device__ __forceinline__ void fwd_groups(const CtaK &p, const CtaState<SM> &S, const FwdLevel &f, unsigned m,
+                                           const Row &row, unsigned long long &sum, bool &ovf) {
+  constexpr int UN = SM ? 2 : 4;  // arcs of a lane in flight
+  const int lane = lane_id(), sub = lane & (W - 1);
+  const uint32_t tp = f.tl - 2u;
+  while (m) {
+    const int src = group_take<W>(m);
+    const int ee = __shfl_sync(BC_FULL, row.e0, src < 0 ? 0 : src);
+    int dg = __shfl_sync(BC_FULL, row.deg, src < 0 ? 0 : src);
+    if (src < 0) dg = 0;
+    const int steps = W == 32 ? dg : (int)__reduce_max_sync(BC_FULL, (unsigned)dg);
+    unsigned long long s = 0ull;
+    bool ov = false;
+    for (int u = 0; u < steps; u += W * UN) {
+      int x[UN];
+      bool nw[UN];
+#pragma unroll
+      for (int k = 0; k < UN; k++) x[k] = u + k * W + sub < dg ? p.ci[ee + u + k * W + sub] : -1;
+      Rec r[UN];
+#pragma unroll
+      for (int k = 0; k < UN; k++) {
+        r[k].tag = f.tl;  // neither a parent nor unreached
+        if (x[k] >= 0) r[k] = cta_rec(S, x[k], tp, false);
+      }
+#pragma unroll
+      for (int k = 0; k < UN; k++) {
+        nw[k] = unreached<SM>(f, r[k].tag) && fwd_claim(S, f, x[k]);
+        if ((r[k].tag & ~1u) == tp) sum_carry(s, ov, r[k].val, r[k].tag & 1u);
+      }
+      fwd_append<SM, UN>(S, f, nw, x);
+    }
+#pragma unroll
+    for (int o = W / 2; o >= 1; o >>= 1) sum_carry(s, ov, __shfl_xor_sync(BC_FULL, s, o), false);
+    const unsigned om = __ballot_sync(BC_FULL, ov);
+    // to the owners: the k-th set bit of m took group k's sum
+    const int k = __popc(m & lanemask_lt());
+    const unsigned long long sk = __shfl_sync(BC_FULL, s, (k * W) & 31);
+    if (((m >> lane) & 1u) && k < 32 / W) {
+      sum = sk;
+      ovf = W == 32 ? om != 0u : ((om >> (k * W)) & ((1u << (W & 31)) - 1u)) != 0u;
+    }
+    m = group_drop<W>(m);
+  }
+}
+
+// Extended-range sigma of the lanes' vertices with ov (rows beyond kThin, or not in registers any
+// more): the sum over the parents in arc order; rows beyond LD by whole warps, lanes in arc
+// order and a fixed-order reduction.
+template <bool SM, int LD>
+__device__ __noinline__ XS fwd_extended(const CtaK &p, CtaState<SM> S, Row row, uint32_t tp, bool ext, bool ov) {
+  XS a;
+  a.m = 0.0;
+  a.e = 0;
+  const int lane = lane_id();
+  if (ov && row.deg <= LD) {
+    for (int u = 0; u < row.deg; u += 4) {
+      int x[4];
+      row_arcs<SM>(p, row, u, row.deg, x);
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        if (x[j] < 0) continue;
+        const Rec r = cta_rec(S, x[j], tp, ext);
+        if ((r.tag & ~1u) == tp) xs_add(a, rec_sigma(r));
+      }
+    }
+  }
+  unsigned m = LD > kNarrowDeg ? __ballot_sync(BC_FULL, ov && row.deg > LD) : 0u;
+  while (m) {
+    const int src = __ffs(m) - 1;
+    m &= m - 1;
+    const int ee = __shfl_sync(BC_FULL, row.e0, src), dg = __shfl_sync(BC_FULL, row.deg, src);
+    XS b;
+    b.m = 0.0;
+    b.e = 0;
+    for (int u = lane; u < dg; u += 32) {
+      const Rec r = cta_rec(S, p.ci[ee + u], tp, ext);
+      if ((r.tag & ~1u) == tp) xs_add(b, rec_sigma(r));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+      XS c;
+      c.m = __shfl_xor_sync(BC_FULL, b.m, o);
+      c.e = __shfl_xor_sync(BC_FULL, b.e, o);
+      xs_add(b, c);
+    }
+    if (lane == src) a = b;
+  }
+  return xs_norm(a);
+}
+
+// Forward sweep from s (Alg. 2 / Alg. 3, one CTA barrier per level).  Returns the deepest
+// non-empty level; *qtot = reached vertices.
+template <bool SM, int LD>
+__device__ __forceinline__ int cta_forward(const CtaK &p, const CtaState<SM> &S, int s, CtaShared &sh,
+                                           int32_t (*ring)[kRing], int *qtot) {
+  const int tid = threadIdx.x, slot = cta_slot(p);
+  const bool xp = p.out_depth != nullptr;
+  FwdLevel f;
+  if constexpr (SM)
+    f.t0 = 0u;
+  else
+    f.t0 = S.base << 1;
+  f.tl = f.t0;
+  bool ext = false;  // some sigma of this source passed 2^64
+  __syncthreads();   // the previous source is done with the state and the counters
   if (tid == 0) {
-    S.d[s] = 0;
-    S.sig[s] = 1ull;
-    S.Q[0] = s;
+    if constexpr (SM) {
+      S.val[s] = 1ull;
+      S.tag[s] = 0;
+      S.vis[s >> 5] |= 1u << (s & 31);
+      S.Q[0] = (uint16_t)s;
+    } else {
+      Rec r;
+      r.val = 1ull;
+      r.tag = f.t0;
+      r.e = 0;
+      st_rec(S.rec + s, r);
+      ring[0][0] = s;
+    }
     S.loff[0] = 0;
     S.loff[1] = 1;
-    sh.q = 1;
+    sh.cnt[1] = 0;
     sh.ovf = 0;
-    sh.lovf[1] = 0;
   }
   __syncthreads();
-  int level = 1, q0 = 0, q1 = 1;
-  while (q1 > q0) {
-    // discover w from v (the compare-and-swap returns the previous depth) and add sigma
-    auto edge = [&](int w, unsigned long long sv, bool ov) {
-      int dw = *(volatile int32_t *)&S.d[w];
-      if (dw < 0) {
-        const int old = atomicCAS(&S.d[w], -1, level);
-        if (old < 0) {
-          S.Q[atomicAdd(&sh.q, 1)] = w;
-          dw = level;
-        } else {
-          dw = old;
+  int q0 = 0, q1 = 1, l = 0;
+  unsigned arcs = 0;  // of the vertices this thread took (nnz < 2^31)
+  int c1 = 1, c2 = 2, c0 = 0;  // counter slots of levels l + 1, l + 2, l
+  for (;;) {
+    const uint32_t tp = f.tl - 2u, tn = f.tl + 2u;
+    f.ring = SM ? nullptr : ring[(l + 1) & 1];
+    f.q1 = q1;
+    f.cnt = &sh.cnt[c1];
+    if (tid == 0) sh.cnt[c2] = 0;
+    for (int b = q0; b < q1; b += blockDim.x) {
+      const int i = b + slot;
+      const bool in = i < q1;
+      if (!__any_sync(BC_FULL, in)) continue;
+      int w = 0;
+      if (in) w = SM ? (int)S.Q[i] : (i - q0 < kRing ? ring[l & 1][i - q0] : (int)S.Q[i]);
+      const Row row = in ? cta_row<SM>(p, w) : no_row();
+      arcs += (unsigned)row.deg;
+      unsigned long long sum = 0ull;
+      bool ov = false;
+      XS a;
+      a.m = 0.0;
+      a.e = 0;
+      int succ = 0;
+      const int dl = row.deg <= LD ? row.deg : 0;
+      for (int u = 0; __any_sync(BC_FULL, u < dl); u += 4) {
+        int x[4];
+        row_arcs<SM>(p, row, u, dl, x);
+        Rec r[4];
+        bool nw[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          r[j].tag = f.tl;  // neither a parent nor a successor
+          if (u < dl && x[j] >= 0) r[j] = cta_rec(S, x[j], tp, ext);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          const bool un = unreached<SM>(f, r[j].tag);
+          nw[j] = un && fwd_claim(S, f, x[j]);
+          if (!SM && (un || r[j].tag == tn) && u < 8) succ |= 1 << (u + j);
+        }
+        fwd_append<SM, 4>(S, f, nw, x);
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+          if ((r[j].tag & ~1u) == tp) sum_carry(sum, ov, r[j].val, r[j].tag & 1u);
+        if (!SM && ov && !xp && row.deg <= kThin) {
+#pragma unroll
+          for (int j = 0; j < 4; j++)
+            if ((r[j].tag & ~1u) == tp) xs_add(a, rec_sigma(r[j]));
+          a = xs_norm(a);
         }
       }
-      if (dw == level) {
-        const unsigned long long old = atomicAdd(&S.sig[w], sv);
-        if (old + sv < old || ov) {
-          atomicOr(&S.ovf[w >> 5], 1u << (w & 31));
-          sh.ovf = 1;
-          sh.lovf[level & 1] = 1;
-        }
+      if constexpr (LD > kNarrowDeg) {
+        constexpr int GD = LD > kGroupDeg ? LD : kGroupDeg;
+        const unsigned mg = __ballot_sync(BC_FULL, row.deg > LD && row.deg <= GD),
+                       mw = __ballot_sync(BC_FULL, row.deg > GD);
+        if (mg) fwd_groups<SM, 8>(p, S, f, mg, row, sum, ov);
+        if (mw) fwd_groups<SM, 32>(p, S, f, mw, row, sum, ov);
       }
-    };
-    cta_split(
-        p, S.Q, q0, q1, sh,
-        [&](int v) {
-          // one thread: the edges in groups of kStage, each stage's loads and atomics of
-          // the group in flight together
-          const unsigned long long sv = S.sig[v];
-          const bool ov = (S.ovf[v >> 5] >> (v & 31)) & 1u;
-          const int e0 = p.rp[v], e1 = p.rp[v + 1];
-          *arcs += (unsigned long long)(e1 - e0);
-          if (p.in_smem) {  // state in shared memory: loads are cheap, no staging
-            for (int e = e0; e < e1; e++) edge(p.ci[e], sv, ov);
-            return;
-          }
-          for (int e = e0; e < e1; e += kStage) {
-            int w[kStage], dw[kStage];
-#pragma unroll
-            for (int j = 0; j < kStage; j++) w[j] = e + j < e1 ? p.ci[e + j] : -1;
-#pragma unroll
-            for (int j = 0; j < kStage; j++) dw[j] = w[j] >= 0 ? *(volatile int32_t *)&S.d[w[j]] : INT_MAX;
-#pragma unroll
-            for (int j = 0; j < kStage; j++) {
-              if (w[j] < 0 || dw[j] >= 0) continue;
-              const int old = atomicCAS(&S.d[w[j]], -1, level);
-              if (old < 0) {
-                S.Q[atomicAdd(&sh.q, 1)] = w[j];
-                dw[j] = level;
-              } else {
-                dw[j] = old;
-              }
-            }
-            unsigned long long old[kStage];
-#pragma unroll
-            for (int j = 0; j < kStage; j++) old[j] = (w[j] >= 0 && dw[j] == level) ? atomicAdd(&S.sig[w[j]], sv) : 0ull;
-#pragma unroll
-            for (int j = 0; j < kStage; j++) {
-              if (w[j] < 0 || dw[j] != level) continue;
-              if (old[j] + sv < old[j] || ov) {
-                atomicOr(&S.ovf[w[j] >> 5], 1u << (w[j] & 31));
-                sh.ovf = 1;
-                sh.lovf[level & 1] = 1;
-              }
-            }
-          }
-        },
-        [&](int v) {
-          const unsigned long long sv = S.sig[v];
-          const bool ov = (S.ovf[v >> 5] >> (v & 31)) & 1u;
-          const int e0 = p.rp[v], e1 = p.rp[v + 1];
-          if (lane == 0) *arcs += (unsigned long long)(e1 - e0);
-          for (int e = e0 + lane; e < e1; e += 32) edge(p.ci[e], sv, ov);
-        });
-    const int q2 = sh.q;
-    const bool lovf = sh.lovf[level & 1] != 0;
-    if (tid == 0) sh.lovf[(level + 1) & 1] = 0;
-    __syncthreads();
-    if (tid == 0) S.loff[level + 1] = q2;
-    if (lovf) {
-      // extended-range sigma of the overflowed vertices of this level: the sum over the
-      // parents (level - 1) in edge order (warps: lanes in edge order, then a fixed-order
-      // reduction)
-      cta_split(
-          p, S.Q, q1, q2, sh,
-          [&](int w) {
-            if (!((S.ovf[w >> 5] >> (w & 31)) & 1u)) return;
-            XS acc;
-            acc.m = 0.0;
-            acc.e = 0;
-            const int e1 = p.rp[w + 1];
-            for (int e = p.rp[w]; e < e1 && p.in_smem; e++) {
-              const int v = p.ci[e];
-              if (S.d[v] == level - 1) xs_add(acc, cta_sigma(S, v));
-            }
-            for (int e = p.rp[w]; e < e1 && !p.in_smem; e += kStage) {
-              int v[kStage];
-              bool par[kStage];
-              XS x[kStage];
-#pragma unroll
-              for (int j = 0; j < kStage; j++) v[j] = e + j < e1 ? p.ci[e + j] : -1;
-#pragma unroll
-              for (int j = 0; j < kStage; j++) par[j] = v[j] >= 0 && S.d[v[j]] == level - 1;
-#pragma unroll
-              for (int j = 0; j < kStage; j++)
-                if (par[j]) x[j] = cta_sigma(S, v[j]);
-#pragma unroll
-              for (int j = 0; j < kStage; j++)
-                if (par[j]) xs_add(acc, x[j]);
-            }
-            acc = xs_norm(acc);
-            S.xm[w] = acc.m;
-            S.xe[w] = acc.e;
-          },
-          [&](int w) {
-            if (!((S.ovf[w >> 5] >> (w & 31)) & 1u)) return;
-            XS acc;
-            acc.m = 0.0;
-            acc.e = 0;
-            const int e1 = p.rp[w + 1];
-            for (int e = p.rp[w] + lane; e < e1; e += 32) {
-              const int v = p.ci[e];
-              if (S.d[v] == level - 1) xs_add(acc, cta_sigma(S, v));
-            }
-#pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) {
-              XS o;
-              o.m = __shfl_down_sync(BC_FULL, acc.m, off);
-              o.e = __shfl_down_sync(BC_FULL, acc.e, off);
-              xs_add(acc, o);
-            }
-            if (lane == 0) {
-              acc = xs_norm(acc);
-              S.xm[w] = acc.m;
-              S.xe[w] = acc.e;
-            }
-          });
+      const bool xs = ov && !xp && (SM || row.deg > kThin);
+      if (__any_sync(BC_FULL, xs)) {
+        const XS y = fwd_extended<SM, LD>(p, S, row, tp, ext, xs);
+        if (xs) a = y;
+      }
+      if (in) {
+        if (!SM) S.Q[i] = w | succ << 24;
+        if (l > 0) fwd_commit(S, f, w, sum, ov, xp, a);  // the source keeps sigma = 1
+        if (ov) sh.ovf = 1;
+      }
     }
+    __syncthreads();
+    const int q2 = q1 + sh.cnt[c1];
+    ext = sh.ovf != 0;
+    if (tid == 0) S.loff[l + 2] = q2;
     q0 = q1;
     q1 = q2;
-    level++;
+    if (q1 == q0) break;
+    l++;
+    f.tl = tn;
+    const int t = c0;
+    c0 = c1;
+    c1 = c2;
+    c2 = t;
   }
+  arcs = __reduce_add_sync(BC_FULL, arcs);
+  if (lane_id() == 0 && arcs) atomicAdd(&sh.arcs, (unsigned long long)arcs);
+  if (tid == 0) {
+    sh.reached += (unsigned long long)q1;
+    sh.levels += (unsigned long long)(l + 1);
+    if ((unsigned long long)l > sh.deepest) sh.deepest = (unsigned long long)l;
+    if (ext) sh.ovf_sources++;
+  }
+  __syncthreads();  // loff, and everyone has read the counters
   *qtot = q1;
-  return level - 2;
+  return l;
 }
 
-// Backward sweep of s (Alg. 4 / Alg. 5): sigma of w taken as m 2^e, r stored scaled by 2^e.
-__device__ void cta_backward(const CtaK &p, const CtaState &S, int s, int lmax, double *bcp,
-                             CtaShared &sh) {
-  const int tid = threadIdx.x, lane = tid & 31;
+// ------------------------------------------------------------------ backward
+// Rows beyond LD: the sum of the successors' r (rescaled to the owner's exponent ew).
+template <bool SM, bool EXT, int W>
+__device__ __forceinline__ void bwd_groups(const CtaK &p, const CtaState<SM> &S, unsigned m, const Row &row, int ew,
+                                           uint32_t tn, float2 &sum) {
+  constexpr int UN = 2;
+  const int lane = lane_id(), sub = lane & (W - 1);
+  while (m) {
+    const int src = group_take<W>(m);
+    const int ee = __shfl_sync(BC_FULL, row.e0, src < 0 ? 0 : src);
+    int dg = __shfl_sync(BC_FULL, row.deg, src < 0 ? 0 : src);
+    const int eo = EXT ? __shfl_sync(BC_FULL, ew, src < 0 ? 0 : src) : 0;
+    if (src < 0) dg = 0;
+    float2 acc = make_float2(0.0f, 0.0f);
+    for (int u = sub; u < dg; u += W * UN) {
+      int x[UN];
+#pragma unroll
+      for (int k = 0; k < UN; k++) x[k] = u + k * W < dg ? p.ci[ee + u + k * W] : -1;
+      Rec r[UN];
+#pragma unroll
+      for (int k = 0; k < UN; k++) {
+        r[k].tag = 0u;
+        if (x[k] >= 0) r[k] = cta_rec(S, x[k], tn, EXT);
+      }
+#pragma unroll
+      for (int k = 0; k < UN; k++)
+        if ((r[k].tag & ~1u) == tn) ff_add(acc, EXT ? ff_scale(rec_r(r[k]), eo - r[k].e) : rec_r(r[k]));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = W / 2; o >= 1; o >>= 1) ff_add(acc, ff_shfl_xor(acc, o));
+    const int k = __popc(m & lanemask_lt());
+    const float2 ak = ff_shfl(acc, (k * W) & 31);
+    if (((m >> lane) & 1u) && k < 32 / W) sum = ak;
+    m = group_drop<W>(m);
+  }
+}
+
+// Backward sweep of s (Alg. 4 / Alg. 5).  Queue entries, rows and a vertex's own record do not
+// depend on the level in progress, so the first window of the next level is loaded before
+// the barrier; only the successors' records wait for it.  The BC partial takes a reduction
+// without a result: one update per vertex and source, ordered by the barriers between levels.
+template <bool SM, int LD, bool EXT>
+__device__ __forceinline__ void cta_backward(const CtaK &p, const CtaState<SM> &S, int s, int lmax, double *bcp,
+                                             CtaShared &sh) {
+  const int tid = threadIdx.x, slot = cta_slot(p);
   const float2 wsrc = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[s] : 0ull));
-  for (int dd = lmax; dd >= 1; --dd) {
-    // commit of w from the sum of its successors' r (rescaled to w's exponent)
-    auto commit = [&](int w, const XS &sw, float2 acc) {
-      const float2 mw = ff_mant(sw.m);
-      const float2 om1 = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull));
-      float2 rw = ff_mul(om1, ff_rcp(mw));
-      ff_add(rw, acc);
-      S.r[w] = rw;  // r scaled by 2^e of w
-      const float2 dl = ff_mul(wsrc, ff_mul(mw, acc));
-      if (!ff_zero(dl)) bcp[w] += ff_to(dl);
-    };
-    cta_split(
-        p, S.Q, S.loff[dd], S.loff[dd + 1], sh,
-        [&](int w) {
-          const XS sw = cta_sigma(S, w);
-          float2 acc = make_float2(0.0f, 0.0f);
-          if (dd < lmax && p.in_smem) {
-            for (int e = p.rp[w]; e < p.rp[w + 1]; e++) {
-              const int v = p.ci[e];
-              if (S.d[v] == dd + 1) ff_add(acc, ff_scale(S.r[v], sw.e - cta_exp(S, v)));
-            }
-          } else if (dd < lmax) {
-            const int e1 = p.rp[w + 1];
-            for (int e = p.rp[w]; e < e1; e += kStage) {
-              int v[kStage];
-              bool suc[kStage];
-              float2 x[kStage];
-              int ev[kStage];
+  int hi = S.loff[lmax + 1], lo = S.loff[lmax];
+  int qe = -1;
+  Row row = no_row();
+  Rec own;
+  own.val = 1ull;
+  own.tag = 0u;
+  own.e = 0;
+  uint32_t tl;
+  if constexpr (SM)
+    tl = (uint32_t)lmax << 1;
+  else
+    tl = (S.base + (uint32_t)lmax) << 1;
+  auto fetch = [&](int q, uint32_t t) {
+    if (q != -1) {
+      row = cta_row<SM>(p, q & kIdMask);
+      own = cta_rec(S, q & kIdMask, t, EXT);
+    } else {
+      row.deg = 0;
+    }
+  };
+  if (lmax >= 1 && lo + slot < hi) qe = (int)S.Q[lo + slot];
+  fetch(qe, tl);
+  int nlo = lmax >= 1 ? S.loff[lmax - 1] : 0;
+  for (int dd = lmax; dd >= 1; --dd, tl -= 2u) {
+    const uint32_t tn = tl + 2u;
+    const int nnlo = dd >= 2 ? S.loff[dd - 2] : 0;
+    const int nqe = (dd > 1 && nlo + slot < lo) ? (int)S.Q[nlo + slot] : -1;
+    for (int b = lo; b < hi; b += blockDim.x) {
+      if (b != lo) {
+        qe = b + slot < hi ? (int)S.Q[b + slot] : -1;
+        fetch(qe, tl);
+      }
+      if (!__any_sync(BC_FULL, qe != -1)) continue;
+      const int w = qe & kIdMask;
+      float2 mw, acc = make_float2(0.0f, 0.0f);
+      int ew = 0;
+      if (EXT) {
+        const XS x = rec_sigma(own);
+        mw = ff_mant(x.m);
+        ew = x.e;
+      } else {
+        mw = ff_u64(own.val);
+      }
+      if (dd < lmax) {
+        const int dl = row.deg <= LD ? row.deg : 0;
+        const unsigned succ = SM ? 0u : (unsigned)qe >> 24;
+        for (int u = 0; u < dl; u += 4) {
+          int x[4];
+          row_arcs<SM>(p, row, u, dl, x);
+          Rec r[4];
 #pragma unroll
-              for (int j = 0; j < kStage; j++) v[j] = e + j < e1 ? p.ci[e + j] : -1;
-#pragma unroll
-              for (int j = 0; j < kStage; j++) suc[j] = v[j] >= 0 && S.d[v[j]] == dd + 1;
-#pragma unroll
-              for (int j = 0; j < kStage; j++) {
-                x[j] = suc[j] ? S.r[v[j]] : make_float2(0.0f, 0.0f);
-                ev[j] = suc[j] ? cta_exp(S, v[j]) : 0;
-              }
-#pragma unroll
-              for (int j = 0; j < kStage; j++)
-                if (suc[j]) ff_add(acc, ff_scale(x[j], sw.e - ev[j]));
-            }
+          for (int j = 0; j < 4; j++) {
+            r[j].tag = 0u;  // not a successor
+            if (x[j] >= 0 && (SM || u >= 8 || ((succ >> (u + j)) & 1u))) r[j] = cta_rec(S, x[j], tn, EXT);
           }
-          commit(w, sw, acc);
-        },
-        [&](int w) {
-          const XS sw = cta_sigma(S, w);
-          float2 acc = make_float2(0.0f, 0.0f);
-          if (dd < lmax) {
-            const int e1 = p.rp[w + 1];
-            for (int e = p.rp[w] + lane; e < e1; e += 32) {
-              const int v = p.ci[e];
-              if (S.d[v] == dd + 1) ff_add(acc, ff_scale(S.r[v], sw.e - cta_exp(S, v)));
-            }
 #pragma unroll
-            for (int m = 16; m >= 1; m >>= 1) ff_add(acc, ff_shfl_xor(acc, m));
-          }
-          if (lane == 0) commit(w, sw, acc);
-        });
+          for (int j = 0; j < 4; j++)
+            if ((r[j].tag & ~1u) == tn) ff_add(acc, EXT ? ff_scale(rec_r(r[j]), ew - r[j].e) : rec_r(r[j]));
+        }
+        __syncwarp();
+        if constexpr (LD > kNarrowDeg) {
+          constexpr int GD = LD > kGroupDeg ? LD : kGroupDeg;
+          const unsigned mg = __ballot_sync(BC_FULL, row.deg > LD && row.deg <= GD),
+                         mb = __ballot_sync(BC_FULL, row.deg > GD);
+          if (mg) bwd_groups<SM, EXT, 8>(p, S, mg, row, ew, tn, acc);
+          if (mb) bwd_groups<SM, EXT, 32>(p, S, mb, row, ew, tn, acc);
+        }
+      }
+      if (qe != -1) {
+        const float2 om1 = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull));
+        float2 rw = ff_mul(om1, ff_rcp(mw));
+        ff_add(rw, acc);
+        if constexpr (SM) {
+          S.val[w] = r_bits(rw);
+          if (EXT) S.e[w] = ew;
+        } else if (EXT) {
+          own.val = r_bits(rw);
+          own.e = ew;
+          st_rec(S.rec + w, own);
+        } else {
+          S.rec[w].val = r_bits(rw);
+        }
+        const float2 dl = ff_mul(wsrc, ff_mul(mw, acc));
+        if (!ff_zero(dl)) atomicAdd(bcp + w, ff_to(dl));
+      }
+    }
+    qe = nqe;
+    fetch(qe, tl - 2u);
+    __syncthreads();
+    hi = lo;
+    lo = nlo;
+    nlo = nnlo;
   }
   if (tid == 0 && p.leaf_term && p.omega && p.omega[s] > 0) {
     const double om = (double)p.omega[s];
-    bcp[s] += om * (2.0 * (double)sh.ns - om - 3.0);
+    atomicAdd(bcp + s, om * (2.0 * (double)sh.ns - om - 3.0));
   }
 }
 
 // n_s of Eq. 3: the reached vertices Q[0, qtot) weighted by 1 + omega (a source with
 // omega(s) > 0 only; the sum is an integer, so its order does not matter).  Ends with a barrier.
-__device__ void cta_weighted_size(const CtaK &p, const CtaState &S, int qtot, CtaShared &sh) {
+template <typename QT>
+__device__ __forceinline__ void cta_weighted_size(const CtaK &p, const QT *Q, int qtot, CtaShared &sh) {
   if (threadIdx.x == 0) sh.ns = 0ull;
   __syncthreads();
   unsigned long long part = 0ull;
-  for (int i = threadIdx.x; i < qtot; i += kCtaThreads) part += 1ull + (unsigned long long)p.omega[S.Q[i]];
+  for (int i = threadIdx.x; i < qtot; i += blockDim.x) part += 1ull + (unsigned long long)p.omega[(int)Q[i] & kIdMask];
 #pragma unroll
   for (int m = 16; m >= 1; m >>= 1) part += __shfl_xor_sync(BC_FULL, part, m);
   if ((threadIdx.x & 31) == 0 && part) atomicAdd(&sh.ns, part);
-  __syncthreads();
-}
-
-__device__ void cta_reset(const CtaState &S, int qtot) {
-  __syncthreads();
-  for (int i = threadIdx.x; i < qtot; i += kCtaThreads) {
-    const int w = S.Q[i];
-    S.d[w] = -1;
-    S.sig[w] = 0ull;
-    S.ovf[w >> 5] = 0u;
-  }
   __syncthreads();
 }
 
@@ -423,203 +766,282 @@ __device__ void cta_reset(const CtaState &S, int qtot) {
 // from those of a and b.  For v != c: level_c(v) = 1 + min(level_a(v), level_b(v)) and
 // sigma_c(v) = sigma_a(v), sigma_b(v) or their sum as the smaller level comes from a, from b
 // or from both (Eq. in Sec. 3.4.2, by the Bellman criterion); level_c(c) = 0, sigma_c(c) = 1.
-__device__ __forceinline__ int deg2_level(const CtaState &A, const CtaState &B, int c, int v) {
-  if (v == c) return 0;
-  const int da = A.d[v], db = B.d[v];
-  if (da < 0 && db < 0) return -1;
-  if (da < 0) return db + 1;
-  if (db < 0) return da + 1;
-  return (da < db ? da : db) + 1;
-}
-__device__ __forceinline__ XS deg2_sigma(const CtaState &A, const CtaState &B, int c, int v) {
-  if (v == c) return xs_u64(1ull);
-  const int da = A.d[v], db = B.d[v];
-  if (db < 0 || (da >= 0 && da < db)) return cta_sigma(A, v);
-  if (da < 0 || db < da) return cta_sigma(B, v);
-  XS x = cta_sigma(A, v);
-  xs_add(x, cta_sigma(B, v));
-  return xs_norm(x);
-}
-
-// exponent of sigma_c(v) as m 2^e (v != c)
-__device__ __forceinline__ int deg2_exp(const CtaState &A, const CtaState &B, int v) {
-  const int da = A.d[v], db = B.d[v];
-  if (db < 0 || (da >= 0 && da < db)) return cta_exp(A, v);
-  if (da < 0 || db < da) return cta_exp(B, v);
-  XS x = cta_sigma(A, v);
-  xs_add(x, cta_sigma(B, v));
-  return xs_norm(x).e;
+__device__ __forceinline__ int rec_level(const CtaState<false> &S, const Rec &r) {
+  return r.tag < (S.base << 1) ? -1 : (int)((r.tag >> 1) - S.base);
 }
 
 // Backward sweep of the 2-degree vertex c on its derived DAG, level by level (the dynamic
 // merging of frontiers, Alg. 8 / Alg. 9): c's level D holds the vertices of a's level D - 1
 // whose level from b is not smaller, and those of b's level D - 1 whose level from a is
-// larger.  rc holds c's r values (scaled by 2^e of sigma_c).  On a residual graph (1-degree
+// larger.  C holds c's records as far as the sweep has come: a neighbour is a successor when
+// its record carries the level after, so the states of a and b are read for a vertex's own
+// sigma only.  EXT (sigma of a or b passed 2^64): r scaled by 2^e of sigma_c.  Runs before the
+// backward sweeps of a and b, which replace their sigma.  On a residual graph (1-degree
 // reduction) the leaf weights enter as in cta_backward; c, a and b share a component, so the
 // weighted component size in sh.ns (set for the triple) is also c's.
-__device__ void cta_backward_deg2(const CtaK &p, const CtaState &A, const CtaState &B, int lmaxA, int lmaxB,
-                                  int c, float2 *rc, double *bcp, CtaShared &sh) {
-  const int lane = threadIdx.x & 31;
+template <int LD, bool EXT>
+__device__ __forceinline__ void cta_backward_deg2(const CtaK &p, const CtaState<false> &A, const CtaState<false> &B,
+                                                  const CtaState<false> &C, int lmaxA, int lmaxB, int c, double *bcp,
+                                                  CtaShared &sh) {
+  const int lane = lane_id(), slot = cta_slot(p);
   const int lmax = 1 + (lmaxA > lmaxB ? lmaxA : lmaxB);
   const float2 wsrc = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[c] : 0ull));
-  auto commit = [&](int w, const XS &sw, float2 acc) {
-    const float2 mw = ff_mant(sw.m);
-    const float2 om1 = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull));
-    float2 rw = ff_mul(om1, ff_rcp(mw));
-    ff_add(rw, acc);
-    rc[w] = rw;
-    const float2 dl = ff_mul(wsrc, ff_mul(mw, acc));
-    if (!ff_zero(dl)) bcp[w] += ff_to(dl);
-  };
   for (int D = lmax; D >= 1; --D) {
+    const uint32_t tc = (C.base + (uint32_t)D) << 1, tn = tc + 2u;
 #pragma unroll 1
     for (int side = 0; side < 2; side++) {
-      const CtaState &S = side ? B : A;
-      const int lm = side ? lmaxB : lmaxA;
-      if (D - 1 > lm) continue;
-      // w belongs to c's level D through this side (ties go to a)
-      auto mine = [&](int w) {
-        if (w == c) return false;
-        const int da = A.d[w], db = B.d[w];
-        return side == 0 ? (db < 0 || da <= db) : (da < 0 || db < da);
-      };
-      cta_split(
-          p, S.Q, S.loff[D - 1], S.loff[D], sh,
-          [&](int w) {
-            if (!mine(w)) return;
-            const XS sw = deg2_sigma(A, B, c, w);
-            float2 acc = make_float2(0.0f, 0.0f);
-            const int e1 = p.rp[w + 1];
-            for (int e = p.rp[w]; e < e1; e += kStage2) {
-              int v[kStage2];
-              bool suc[kStage2];
-#pragma unroll
-              for (int j = 0; j < kStage2; j++) v[j] = e + j < e1 ? p.ci[e + j] : -1;
-#pragma unroll
-              for (int j = 0; j < kStage2; j++) suc[j] = v[j] >= 0 && deg2_level(A, B, c, v[j]) == D + 1;
-#pragma unroll
-              for (int j = 0; j < kStage2; j++)
-                if (suc[j]) ff_add(acc, ff_scale(rc[v[j]], sw.e - deg2_exp(A, B, v[j])));
+      if (D - 1 > (side ? lmaxB : lmaxA)) continue;
+      const int32_t *Q = side ? B.Q : A.Q, *loff = side ? B.loff : A.loff;
+      const int i1 = loff[D];
+      for (int b = loff[D - 1]; b < i1; b += blockDim.x) {
+        const int i = b + slot;
+        const int w = i < i1 ? Q[i] & kIdMask : c;
+        bool mine = w != c;
+        Row row = no_row();
+        float2 mw = make_float2(1.0f, 0.0f);
+        int ew = 0;
+        if (mine) {
+          row = cta_row<false>(p, w);
+          const Rec ra = ld_rec(A.rec + w), rb = ld_rec(B.rec + w);
+          const int da = rec_level(A, ra), db = rec_level(B, rb);
+          // w belongs to c's level D through this side (ties go to a)
+          mine = side == 0 ? (db < 0 || da <= db) : (da < 0 || db < da);
+          if (EXT) {
+            XS x = rec_sigma(side ? rb : ra);
+            if (da == db) {
+              xs_add(x, rec_sigma(rb));
+              x = xs_norm(x);
             }
-            commit(w, sw, acc);
-          },
-          [&](int w) {
-            if (!mine(w)) return;
-            const XS sw = deg2_sigma(A, B, c, w);
-            float2 acc = make_float2(0.0f, 0.0f);
-            const int e1 = p.rp[w + 1];
-            for (int e = p.rp[w] + lane; e < e1; e += 32) {
-              const int v = p.ci[e];
-              if (deg2_level(A, B, c, v) != D + 1) continue;
-              ff_add(acc, ff_scale(rc[v], sw.e - deg2_exp(A, B, v)));
+            mw = ff_mant(x.m);
+            ew = x.e;
+          } else {
+            mw = ff_u64(side ? rb.val : ra.val);
+            if (da == db) ff_add(mw, ff_u64(rb.val));
+          }
+        }
+        float2 acc = make_float2(0.0f, 0.0f);
+        if (D < lmax) {
+          const int dl = mine && row.deg <= LD ? row.deg : 0;
+          for (int u = 0; u < dl; u += 4) {
+            int x[4];
+            row_arcs<false>(p, row, u, dl, x);
+            Rec r[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+              r[j].tag = 0u;
+              if (x[j] >= 0) r[j] = ld_rec(C.rec + x[j]);
             }
 #pragma unroll
-            for (int m = 16; m >= 1; m >>= 1) ff_add(acc, ff_shfl_xor(acc, m));
-            if (lane == 0) commit(w, sw, acc);
-          });
+            for (int j = 0; j < 4; j++)
+              if (r[j].tag == tn) ff_add(acc, EXT ? ff_scale(rec_r(r[j]), ew - r[j].e) : rec_r(r[j]));
+          }
+          __syncwarp();
+          unsigned m = LD > kNarrowDeg ? __ballot_sync(BC_FULL, mine && row.deg > LD) : 0u;
+          while (m) {
+            const int src = __ffs(m) - 1;
+            m &= m - 1;
+            const int ee = __shfl_sync(BC_FULL, row.e0, src), dg = __shfl_sync(BC_FULL, row.deg, src),
+                      eo = __shfl_sync(BC_FULL, ew, src);
+            float2 t = make_float2(0.0f, 0.0f);
+            for (int u = lane; u < dg; u += 32) {
+              const Rec r = ld_rec(C.rec + p.ci[ee + u]);
+              if (r.tag == tn) ff_add(t, EXT ? ff_scale(rec_r(r), eo - r.e) : rec_r(r));
+            }
+            __syncwarp();
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) ff_add(t, ff_shfl_xor(t, o));
+            if (lane == src) acc = t;
+          }
+        }
+        if (mine) {
+          const float2 om1 = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull));
+          float2 rw = ff_mul(om1, ff_rcp(mw));
+          ff_add(rw, acc);
+          Rec r;
+          r.val = r_bits(rw);
+          r.tag = tc;
+          r.e = ew;
+          st_rec(C.rec + w, r);
+          const float2 dl = ff_mul(wsrc, ff_mul(mw, acc));
+          if (!ff_zero(dl)) atomicAdd(bcp + w, ff_to(dl));
+        }
+      }
     }
+    __syncthreads();
   }
   if (threadIdx.x == 0 && p.leaf_term && p.omega && p.omega[c] > 0) {
     const double om = (double)p.omega[c];
-    bcp[c] += om * (2.0 * (double)sh.ns - om - 3.0);
+    atomicAdd(bcp + c, om * (2.0 * (double)sh.ns - om - 3.0));
   }
 }
 
-__global__ void __launch_bounds__(kCtaThreads, 2) k_cta_sources(CtaK p) {
+// SM: state in shared memory; TRI: 2-degree triples (a second state, both in global memory).
+template <bool SM, bool TRI, int MAXT, int LD>
+__global__ void __launch_bounds__(MAXT, 1) k_cta_sources(CtaK p) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = p.n;
-  const int tid = threadIdx.x, lane = tid & 31;
-  char *gslice = p.gws + (size_t)blockIdx.x * p.slice;
-  const size_t sb = cta_state_bytes(n), xb = cta_extra_bytes(n);
-  // state A: shared memory when it fits; state B and c's r (2-degree triples) after it
-  char *g = gslice;
-  char *blkA = p.in_smem ? (char *)smem : g;
-  if (!p.in_smem) g += sb;
-  const CtaState A = cta_carve(blkA, g, n);
-  g += xb;
-  CtaState B = A;
-  float2 *rc = nullptr;
-  if (p.ntri) {
-    B = cta_carve(g, g + sb, n);
-    rc = (float2 *)(g + sb + xb);
+  const int tid = threadIdx.x;
+  uint32_t *hdr = (uint32_t *)(p.gws + (size_t)blockIdx.x * p.slice);  // the states' bases
+  char *g = (char *)hdr + 16;
+  // shared memory: the state, or the ring of the last two levels' entries
+  int32_t(*ring)[kRing] = SM ? nullptr : (int32_t(*)[kRing])smem;
+  CtaState<SM> A = cta_carve<SM>((char *)smem, g, n);
+  CtaState<SM> B = A;  // TRI only
+  CtaState<SM> C = A;  // TRI only: c's records
+  if constexpr (TRI) {
+    B = cta_carve<SM>(nullptr, g + cta_state_bytes(n, false), n);
+    C.rec = (Rec *)(g + 2 * cta_state_bytes(n, false));
   }
   double *bcp = p.bcp + (size_t)blockIdx.x * n;
   __shared__ CtaShared sh;
 
-  for (int v = tid; v < n; v += kCtaThreads) bcp[v] = 0.0;
-  if (tid == 0) sh.nbig = 0;  // the big-vertex list of cta_split starts empty
-  // every source resets the vertices it reached, so state in global memory stays clean from
-  // one call to the next; shared memory starts undefined
-  if (p.in_smem || !p.clean) cta_clear(A, n);
-  if (p.ntri && !p.clean) cta_clear(B, n);
-  unsigned long long my_arcs = 0, my_reached = 0, my_levels = 0, my_deep = 0, my_ovf = 0;
+  for (int v = tid; v < n; v += blockDim.x) bcp[v] = 0.0;
+  // records of earlier sources and calls read as not reached below the base
+  if constexpr (SM) {
+    cta_clear(A, n);
+  } else {
+    if (!p.clean) {
+      cta_clear(A, n);
+      if (TRI) cta_clear(B, n);
+      if (TRI) cta_clear(C, n);
+    } else {
+      A.base = hdr[0];
+      if (TRI) B.base = hdr[1];
+      if (TRI) C.base = hdr[2];
+    }
+  }
+  if (tid == 0) sh.arcs = sh.reached = sh.levels = sh.deepest = sh.ovf_sources = 0ull;
   __syncthreads();
 
-  auto account = [&](int lmax, int qtot) {
-    my_reached += (unsigned long long)qtot;
-    my_levels += (unsigned long long)(lmax + 1);
-    if ((unsigned long long)lmax > my_deep) my_deep = (unsigned long long)lmax;
-    if (sh.ovf) my_ovf++;
+  auto done_with = [&](CtaState<SM> &S, int lmax) {
+    if constexpr (SM) {
+      __syncthreads();
+      cta_clear(S, n);
+    } else {  // the levels just used are behind the next base
+      S.base += (uint32_t)lmax + 2u;
+      if (S.base > kBaseMax) {
+        __syncthreads();
+        cta_clear(S, n);
+      }
+    }
   };
   int s0 = (int)blockIdx.x, s1 = p.nsrc, sstep = (int)gridDim.x;
-  if (p.nreq > 0) {  // the sources of this CTA's request, strided over the request's CTAs
-    const int32_t *rc = p.req + p.nreq + 1;
+  if (!TRI && p.nreq > 0) {  // the sources of this CTA's request, strided over the request's CTAs
+    const int32_t *rcta = p.req + p.nreq + 1;
     int q = 0;
-    while (q + 1 < p.nreq && (int)blockIdx.x >= rc[q + 1]) q++;
-    s0 = p.req[q] + ((int)blockIdx.x - rc[q]);
+    while (q + 1 < p.nreq && (int)blockIdx.x >= rcta[q + 1]) q++;
+    s0 = p.req[q] + ((int)blockIdx.x - rcta[q]);
     s1 = p.req[q + 1];
-    sstep = rc[q + 1] - rc[q];
+    sstep = rcta[q + 1] - rcta[q];
   }
-  for (int si = s0; si < s1; si += sstep) {
-    const int s = p.src[si];
-    int qtot = 0;
-    const int lmax = cta_forward(p, A, s, sh, &qtot, &my_arcs);
-    account(lmax, qtot);
-    if (p.leaf_term && p.omega && p.omega[s] > 0) cta_weighted_size(p, A, qtot, sh);
-    if (p.out_depth) {  // forward-only export (sssp of src[0])
-      for (int v = tid; v < n; v += kCtaThreads) {
-        p.out_depth[v] = A.d[v];
-        p.out_sigma[v] = A.sig[v];
-        p.out_ovf[v] = (uint8_t)((A.ovf[v >> 5] >> (v & 31)) & 1u);
+  if constexpr (!TRI) {
+    for (int si = s0; si < s1; si += sstep) {
+      const int s = p.src[si];
+      int qtot = 0;
+      const int lmax = cta_forward<SM, LD>(p, A, s, sh, ring, &qtot);
+      if (p.leaf_term && p.omega && p.omega[s] > 0) cta_weighted_size(p, A.Q, qtot, sh);
+      if (p.out_depth) {  // forward-only export (sssp of src[0])
+        for (int v = tid; v < n; v += blockDim.x) {
+          int d = -1;
+          unsigned long long x = 0ull;
+          uint32_t t;
+          if constexpr (SM) {
+            t = A.tag[v];
+            if (t != kSmFree) {
+              d = (int)(t >> 1);
+              x = A.val[v];
+            }
+          } else {
+            const Rec r = ld_rec(A.rec + v);
+            t = r.tag;
+            if (t >= (A.base << 1)) {
+              d = (int)((t >> 1) - A.base);
+              x = r.val;
+            }
+          }
+          p.out_depth[v] = d;
+          p.out_sigma[v] = x;
+          p.out_ovf[v] = d >= 0 ? (uint8_t)(t & 1u) : (uint8_t)0;
+        }
+      } else if (sh.ovf) {
+        cta_backward<SM, LD, true>(p, A, s, lmax, bcp, sh);
+      } else {
+        cta_backward<SM, LD, false>(p, A, s, lmax, bcp, sh);
       }
-    } else {
-      cta_backward(p, A, s, lmax, bcp, sh);
+      done_with(A, lmax);
     }
-    cta_reset(A, qtot);
+  } else {
+    // single sources, then the 2-degree triples (a, b, c): a and b as usual, c from their two
+    // DAGs before their backward sweeps replace sigma by r
+    for (int u = blockIdx.x; u < p.nsrc + p.ntri; u += gridDim.x) {
+      const bool tri = u >= p.nsrc;
+      const int ti = 3 * (u - p.nsrc);
+      const int va = tri ? p.tri[ti] : p.src[u], vb = tri ? p.tri[ti + 1] : 0, vc = tri ? p.tri[ti + 2] : 0;
+      int la = 0, lb = 0, qtot = 0, xa = 0, xb = 0;
+#pragma unroll 1
+      for (int k = 0; k <= (int)tri; k++) {
+        const int l = cta_forward<SM, LD>(p, k ? B : A, k ? vb : va, sh, ring, &qtot);
+        if (k) {
+          lb = l;
+          xb = sh.ovf;
+        } else {
+          la = l;
+          xa = sh.ovf;
+        }
+      }
+      // a, b and c share a component: one weighted size (of the state run last) serves all three
+      if (p.leaf_term && p.omega && (p.omega[va] > 0 || (tri && (p.omega[vb] > 0 || p.omega[vc] > 0))))
+        cta_weighted_size(p, tri ? B.Q : A.Q, qtot, sh);
+      if (tri) {
+        if (xa | xb)
+          cta_backward_deg2<LD, true>(p, A, B, C, la, lb, vc, bcp, sh);
+        else
+          cta_backward_deg2<LD, false>(p, A, B, C, la, lb, vc, bcp, sh);
+        done_with(C, 1 + max(la, lb));
+      }
+#pragma unroll 1
+      for (int k = 0; k <= (int)tri; k++) {
+        if (k ? xb : xa)
+          cta_backward<SM, LD, true>(p, k ? B : A, k ? vb : va, k ? lb : la, bcp, sh);
+        else
+          cta_backward<SM, LD, false>(p, k ? B : A, k ? vb : va, k ? lb : la, bcp, sh);
+      }
+      done_with(A, la);
+      if (tri) done_with(B, lb);
+    }
   }
-  // 2-degree triples (a, b, c): a and b as usual, c from their two DAGs
-  for (int ti = blockIdx.x; ti < p.ntri; ti += gridDim.x) {
-    const int a = p.tri[3 * ti], b = p.tri[3 * ti + 1], c = p.tri[3 * ti + 2];
-    int qa = 0, qb = 0;
-    const int la = cta_forward(p, A, a, sh, &qa, &my_arcs);
-    account(la, qa);
-    // a, b and c share a component: one weighted size serves all three
-    if (p.leaf_term && p.omega && (p.omega[a] > 0 || p.omega[b] > 0 || p.omega[c] > 0))
-      cta_weighted_size(p, A, qa, sh);
-    cta_backward(p, A, a, la, bcp, sh);
-    const int lb = cta_forward(p, B, b, sh, &qb, &my_arcs);
-    account(lb, qb);
-    cta_backward(p, B, b, lb, bcp, sh);
-    cta_backward_deg2(p, A, B, la, lb, c, rc, bcp, sh);
-    cta_reset(A, qa);
-    cta_reset(B, qb);
-  }
-  // statistics
-  for (int m = 16; m >= 1; m >>= 1) my_arcs += __shfl_xor_sync(BC_FULL, my_arcs, m);
-  if (lane == 0 && my_arcs) atomicAdd(&p.stats[1], my_arcs);
+  __syncthreads();
   if (tid == 0) {
-    atomicAdd(&p.stats[0], my_reached);
-    atomicAdd(&p.stats[2], my_levels);
-    atomicMax(&p.stats[3], my_deep);
-    if (my_ovf) atomicAdd(&p.stats[4], my_ovf);
+    if constexpr (!SM) {
+      hdr[0] = A.base;
+      if (TRI) hdr[1] = B.base;
+      if (TRI) hdr[2] = C.base;
+    }
+    atomicAdd(&p.stats[0], sh.reached);
+    atomicAdd(&p.stats[1], sh.arcs);
+    atomicAdd(&p.stats[2], sh.levels);
+    atomicMax(&p.stats[3], sh.deepest);
+    if (sh.ovf_sources) atomicAdd(&p.stats[4], sh.ovf_sources);
   }
 }
 
-// bc[v] += sum over CTAs c (in order) of bcp[c][v]
+// bc[v] += sum over CTAs c (in order) of bcp[c][v]; sixteen partials in flight at a time
+__device__ __forceinline__ double cta_partials(const double *bcp, int c0, int c1, int n, int v) {
+  double sum = 0.0;
+  int c = c0;
+  for (; c + 16 <= c1; c += 16) {
+    double x[16];
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = bcp[(size_t)(c + k) * n + v];
+#pragma unroll
+    for (int k = 0; k < 16; k++) sum += x[k];
+  }
+  for (; c < c1; c++) sum += bcp[(size_t)c * n + v];
+  return sum;
+}
 __global__ void k_cta_reduce(const double *bcp, int ncta, int n, double *bc) {
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    double sum = 0.0;
-    for (int c = 0; c < ncta; c++) sum += bcp[(size_t)c * n + v];
+    const double sum = cta_partials(bcp, 0, ncta, n, v);
     if (sum != 0.0) bc[v] += sum;
   }
 }
@@ -629,8 +1051,7 @@ __global__ void k_cta_reduce(const double *bcp, int ncta, int n, double *bc) {
 __global__ void k_cta_reduce_req(const double *bcp, int nreq, const int32_t *rc, double *const *req_bc, int n) {
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
     for (int q = 0; q < nreq; q++) {
-      double sum = 0.0;
-      for (int c = rc[q]; c < rc[q + 1]; c++) sum += bcp[(size_t)c * n + v];
+      const double sum = cta_partials(bcp, rc[q], rc[q + 1], n, v);
       if (sum != 0.0) req_bc[q][v] += sum;
     }
   }
@@ -639,11 +1060,13 @@ __global__ void k_cta_reduce_req(const double *bcp, int nreq, const int32_t *rc,
 }  // namespace
 
 struct CtaWS {
-  int n = 0, ncta = 0, in_smem = 0, tri = 0;
-  bool clean = false;  // global-memory state left cleared by a completed launch
-  size_t slice = 0, smem = 0;
+  int n = 0, ncta = 0;
+  int kind = -1;       // slice layout of the last completed launch: 0 global, 1 shared, 2 triples
+  bool clean = false;  // the slices' bases and records are valid for that layout
+  size_t slice = 0;    // bytes per CTA
   double *bcp = nullptr;
   char *gws = nullptr;
+  int4 *row4 = nullptr;  // row records (null: they did not fit the HBM budget)
   unsigned long long *stats = nullptr;
   int32_t *req = nullptr;  // request offsets of a launch with several requests
   size_t bytes = 0;
@@ -653,18 +1076,62 @@ void cta_free(Ctx *ctx, CtaWS *ws) {
   if (!ws) return;
   cudaFree(ws->bcp);
   cudaFree(ws->gws);
+  cudaFree(ws->row4);
   cudaFree(ws->stats);
   cudaFree(ws->req);
   ctx->mem.release(nullptr, ws->bytes);
   delete ws;
 }
 
-static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, bool tri) {
-  CtaWS *ws = *wsp;
-  const size_t st = cta_state_bytes(n);
-  const int in_smem = st <= kCtaSmemMax;
-  const size_t smem = in_smem ? st : 0;
-  int bps = 0;
+// How a call runs: state in shared memory or not, threads per CTA, CTAs of the whole GPU.
+struct CtaPlan {
+  int kind = 0, threads = 512, ncta = 0;
+  size_t smem = 0;
+  const void *kernel = nullptr;
+};
+
+// The rule, and both sides of its lines (ms per call, this GPU):
+// * State in shared memory where it fits (n <= 22,654): G(n, 4n) n = 16,384, 500 sources 1.15
+//   against 1.79 from global memory, social graph n = 20,001, 3000 sources 9.9 against 16.3.
+//   Narrow graphs (largest degree <= 8, road-like: levels of about sqrt(n) vertices) only while
+//   three CTAs' states fit an SM: their levels leave a large CTA idle, so many small CTAs win
+//   (roads with chains, all sources: n = 9,600 7.2 from global memory with eight CTAs per SM,
+//   18 with one state per SM; n = 4,900 2.6 from shared, 2.7 from global memory).
+// * 64 registers and 1024 threads per SM where rows beyond 64 arcs keep whole warps busy (R-MAT
+//   scale 12 all sources 3.3 against 4.1 with 128 registers and 512 threads; social graph above
+//   10.0 against 10.7), else 128 registers and 512 threads (G(9000, 36,000) all sources 9.0
+//   against 10.0), a lane then taking rows of up to 32 arcs instead of 16 (G(9000, 72,000):
+//   12.9 against 16.4).  From global memory 128 registers (64 spill in the sweeps: grid 1024^2
+//   92 against 70); narrow graphs need no code for larger rows and run with 80 (59).
+// * Threads: an SM's threads over the states that fit it and have a source (one source on
+//   n = 1000: 85 us with 512, 95 with 128); from global memory 512 (social graph
+//   n = 60,001, 500 sources: 11.9, 13.3 with 256), narrow graphs 96 / 192 / 384 by size (grid
+//   300^2, 500 sources: 5.5 with 192, 6.7 with 128; grid 1024^2: 59 with 384, 88 with 256).
+static bc_status cta_plan(Ctx *ctx, int n, int max_degree, int units, bool tri, CtaPlan *pl) {
+  const bool narrow = max_degree > 0 && max_degree <= kNarrowDeg;
+  const bool fits = !tri && n < (1 << 15) && cta_smem_bytes(n, false) <= kCtaSmemMax;
+  // CTAs whose state fits an SM's shared memory (1 KB per CTA is the system's, the rest static)
+  const int per_sm = fits ? (int)((size_t)227 * 1024 / (cta_smem_bytes(n, cta_smem_q(n)) + 1280)) : 0;
+  const bool sm = fits && (!narrow || per_sm >= 3);
+  const int lb = sm && max_degree > 64 ? 1024 : 512;
+  pl->kind = tri ? 2 : sm ? 1 : 0;
+  if (tri)
+    pl->kernel = narrow ? (const void *)k_cta_sources<false, true, 512, kNarrowDeg>
+                        : (const void *)k_cta_sources<false, true, 512, 16>;
+  else if (!sm)
+    pl->kernel = narrow ? (const void *)k_cta_sources<false, false, 768, kNarrowDeg>
+                        : (const void *)k_cta_sources<false, false, 512, 16>;
+  else if (narrow)
+    pl->kernel = (const void *)k_cta_sources<true, false, 640, kNarrowDeg>;
+  else
+    pl->kernel = lb == 512 ? (const void *)k_cta_sources<true, false, 512, 32>
+                           : (const void *)k_cta_sources<true, false, 1024, 16>;
+  pl->smem = sm ? cta_smem_bytes(n, cta_smem_q(n)) : sizeof(int32_t) * 2 * kRing;
+  const int busy = std::min(per_sm, (units + ctx->num_sms - 1) / ctx->num_sms);  // CTAs per SM in use
+  if (sm)
+    pl->threads = narrow ? std::max(64, 640 / std::min(per_sm, 8) & ~31) : std::max(128, lb / std::min(busy, 8) & ~31);
+  else
+    pl->threads = !narrow ? 512 : n < 16384 ? 96 : n < 500000 ? (tri ? 128 : 192) : 384;
   {
     // the attribute is per function and device: set it once, to the largest size used, so
     // that concurrent callers (serving workers on graphs of different sizes) never lower it
@@ -675,20 +1142,30 @@ static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, bool tri) {
     BC_CUDA_TRY(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(mu);
     if (dev < 0 || dev >= 64 || !done[dev]) {
-      BC_CUDA_TRY(cudaFuncSetAttribute(k_cta_sources, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kCtaSmemMax));
+      for (const void *k : {(const void *)k_cta_sources<true, false, 640, kNarrowDeg>,
+                            (const void *)k_cta_sources<true, false, 512, 32>,
+                            (const void *)k_cta_sources<true, false, 1024, 16>})
+        BC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtaSmemMax));
       if (dev >= 0 && dev < 64) done[dev] = true;
     }
   }
-  BC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_cta_sources, kCtaThreads, smem));
+  int bps = 0;
+  BC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, pl->kernel, pl->threads, pl->smem));
   if (bps < 1) return fail(BC_ECUDA, "CTA per-source kernel does not fit on an SM");
-  if (!in_smem) bps = std::min(bps, 2);  // slices live in L2 / HBM: keep their total small
-  int ncta = ctx->num_sms * bps;
-  // slice: state A (unless in shared memory) and its extras; with triples also state B,
-  // its extras and c's r values
-  const size_t slice = ((in_smem ? 0 : st) + cta_extra_bytes(n) +
-                        (tri ? st + cta_extra_bytes(n) + (size_t)n * 8 : 0) + 255) & ~(size_t)255;
+  pl->ncta = ctx->num_sms * bps;
+  return BC_OK;
+}
+
+// A workspace of min(plan's CTAs, CTAs the call can use) slices for graphs of n vertices.
+static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, int64_t units, const CtaPlan &pl) {
+  CtaWS *ws = *wsp;
+  // sizes of the largest layout (with triples only once a call has them)
+  const bool tri = pl.kind == 2;
+  size_t slice = 16 + cta_state_bytes(n, false) * (tri ? 2 : 1) + (tri ? (size_t)n * 16 : 0);
+  if (pl.kind == 1) slice = 16 + cta_state_bytes(n, true);
+  slice = (slice + 255) & ~(size_t)255;
   const size_t per_cta = (size_t)n * 8 + slice;
+  int ncta = (int)std::min<int64_t>(pl.ncta, std::max<int64_t>(units, 32));
   if (ctx->mem.budget) {  // fewer CTAs when the context's HBM budget is tight: at most half
     // of what is free, so that requests arriving meanwhile still find room (serving)
     const size_t used = ctx->mem.used.load() - (ws ? ws->bytes : 0);
@@ -696,19 +1173,17 @@ static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, bool tri) {
     ncta = (int)std::min<size_t>((size_t)ncta, std::max<size_t>(avail / 2 / per_cta, avail >= per_cta ? 1 : 0));
     if (ncta < 1) return fail(BC_ENOMEM, "CTA per-source workspace exceeds the context HBM budget");
   }
-  if (ws && ws->n == n && ws->ncta == ncta && ws->tri >= (int)tri) return BC_OK;
+  if (ws && ws->n == n && ws->ncta >= ncta && ws->slice >= slice) return BC_OK;
   if (ws) {
     cta_free(ctx, ws);
     *wsp = nullptr;
   }
-  ws = new CtaWS();
+  ws = new (std::nothrow) CtaWS();
+  if (!ws) return fail(BC_ENOMEM, "host allocation failed");
   ws->n = n;
   ws->ncta = ncta;
-  ws->in_smem = in_smem;
-  ws->smem = smem;
   ws->slice = slice;
-  ws->tri = tri ? 1 : 0;
-  const size_t b_bcp = (size_t)ncta * n * 8, b_gws = ws->slice * ncta;
+  const size_t b_bcp = (size_t)ncta * n * 8, b_gws = slice * ncta, b_row = pl.kind == 1 ? 0 : (size_t)n * 16;
   ws->bytes = b_bcp + b_gws + 64 + 2 * (kCtaMaxReq + 1) * sizeof(int32_t);
   bc_status s = ctx->mem.alloc(nullptr, ws->bytes);
   if (s) {
@@ -724,6 +1199,17 @@ static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, bool tri) {
     cta_free(ctx, ws);
     return fail(BC_ENOMEM, "CTA per-source workspace allocation failed");
   }
+  // row records where the budget leaves room (the kernel reads rp and ci without them)
+  if (b_row && (!ctx->mem.budget || ctx->mem.used.load() + 4 * b_row < ctx->mem.budget) &&
+      ctx->mem.alloc(nullptr, b_row) == BC_OK) {
+    if (cudaMalloc((void **)&ws->row4, b_row) == cudaSuccess) {
+      ws->bytes += b_row;
+    } else {
+      cudaGetLastError();
+      ws->row4 = nullptr;
+      ctx->mem.release(nullptr, b_row);
+    }
+  }
   *wsp = ws;
   return BC_OK;
 }
@@ -735,10 +1221,13 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   const int n = dg->n;
   const bool sssp = a.out_depth != nullptr;
   if (a.nsrc <= 0 && a.ntri <= 0) return BC_OK;
-  bc_status s = cta_ensure(ctx, wsp, n, a.ntri > 0);
+  CtaPlan pl;
+  const int units = sssp ? 1 : std::max(a.nsrc, a.ntri);
+  bc_status s = cta_plan(ctx, n, a.max_degree, units, !sssp && a.ntri > 0, &pl);
+  if (!s) s = cta_ensure(ctx, wsp, n, units, pl);
   if (s) return s;
   CtaWS *ws = *wsp;
-  (void)g;
+  const int max_cta = std::min(pl.ncta, ws->ncta);
   CtaK p;
   memset(&p, 0, sizeof(p));
   p.n = n;
@@ -751,8 +1240,8 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   p.bcp = ws->bcp;
   p.gws = ws->gws;
   p.slice = ws->slice;
-  p.in_smem = ws->in_smem;
-  p.clean = ws->clean ? 1 : 0;
+  p.row4 = pl.kind == 1 ? nullptr : ws->row4;
+  p.spread = a.max_degree <= 0 || a.max_degree > kThin;
   p.stats = ws->stats;
   p.out_depth = a.out_depth;
   p.out_sigma = a.out_sigma;
@@ -762,7 +1251,7 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   if (a.nreq > 0 && (sssp || p.ntri || a.nreq > kCtaMaxReq || !a.h_req_k || !a.req_bc))
     return fail(BC_EINVAL, "CTA per-source kernel: bad request list");
   // requests per launch: groups of consecutive requests, each request with CTAs of its own
-  // (at most ws->ncta requests per launch)
+  // (at most max_cta requests per launch)
   std::vector<std::vector<int32_t>> hreq;
   int nlaunch = 0, launched_max = 0;
   BC_CUDA_TRY(cudaMemsetAsync(ws->stats, 0, 64, st));
@@ -770,14 +1259,15 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   BC_CUDA_TRY(cudaEventCreate(&e0));
   BC_CUDA_TRY(cudaEventCreate(&e1));
   cudaEventRecord(e0, st);
-  const bool was_clean = ws->clean;
+  const bool was_clean = ws->clean && ws->kind == pl.kind;
   ws->clean = false;  // until the launches are known to have completed
+  if (p.row4) k_cta_rows<<<ctx->num_sms * 4, 256, 0, st>>>(n, dg->rp, dg->ci, ws->row4);
   cudaError_t le = cudaSuccess;
   auto launch = [&](const CtaK &kp, int ncta, const int32_t *rc, double *const *rbc) {
     CtaK q = kp;
     q.clean = (was_clean || launched_max >= ncta) ? 1 : 0;
-    k_cta_sources<<<ncta, kCtaThreads, ws->smem, st>>>(q);
-    le = cudaGetLastError();
+    void *args[] = {&q};
+    le = cudaLaunchKernel(pl.kernel, dim3(ncta), dim3(pl.threads), args, pl.smem, st);
     launched_max = std::max(launched_max, ncta);
     nlaunch++;
     if (le == cudaSuccess && !sssp && q.nreq > 0) {
@@ -789,15 +1279,15 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
     }
   };
   if (a.nreq <= 0) {
-    launch(p, std::max(1, std::min(ws->ncta, std::max(p.nsrc, p.ntri))), nullptr, nullptr);
+    launch(p, std::max(1, std::min(max_cta, std::max(p.nsrc, p.ntri))), nullptr, nullptr);
   } else {
     int q0 = 0, soff = 0;
     while (q0 < a.nreq && le == cudaSuccess) {
-      const int q1 = std::min(a.nreq, q0 + ws->ncta);
+      const int q1 = std::min(a.nreq, q0 + max_cta);
       const int R = q1 - q0;
       long long K = 0;
       for (int q = q0; q < q1; q++) K += a.h_req_k[q];
-      const int C = (int)std::max<long long>(R, std::min<long long>(ws->ncta, K));
+      const int C = (int)std::max<long long>(R, std::min<long long>(max_cta, K));
       // CTAs in proportion to the sources (at least one each, at most one per source), then
       // the rest, one at a time, to the request with the most rounds of sources per CTA
       std::vector<int> c(R);
@@ -866,6 +1356,7 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   BC_CUDA_TRY(cudaStreamSynchronize(st));
   // the launched CTAs left their state cleared; CTAs not launched kept theirs
   ws->clean = was_clean || launched_max == ws->ncta;
+  ws->kind = pl.kind;
   if (acc) {
     acc->seconds += ms * 1e-3;
     acc->sources += p.nsrc + 3ll * p.ntri;
@@ -874,7 +1365,7 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
     acc->reached_arcs += (int64_t)hs[1];
     acc->levels += (int64_t)hs[2];
     if ((int32_t)hs[3] > acc->max_depth) acc->max_depth = (int32_t)hs[3];
-    acc->kernel_launches += sssp ? nlaunch : 2 * nlaunch;
+    acc->kernel_launches += (sssp ? nlaunch : 2 * nlaunch) + (p.row4 ? 1 : 0);
     if (acc->tile_width == 0) acc->tile_width = 1;
   }
   return BC_OK;
