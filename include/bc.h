@@ -248,9 +248,9 @@ const char *bc_version(void);
  * BC_NOALLOC_MAX_N vertices, that every GPU loading the library holds until the process
  * exits; the CUDA runtime places it on a device when it loads the library's device code
  * there (with lazy module loading: at the latest during the first call on that device),
- * and no call allocates anything.  The call clears that array at its start, checks every
- * source id on the device, and synchronises cuda_stream twice (after the check and after
- * the traversal): it returns when the result is complete.  Calls in one process share the
+ * and no call allocates anything.  The call clears the part of that array it uses, checks every
+ * source id on the device, and synchronises cuda_stream (after the traversal, on larger graphs
+ * also after the check): it returns when the result is complete.  Calls in one process share the
  * array and are serialised (one runs at a time, to completion); each process has its own
  * copy of it, so calls in different processes never share it.  The first call on a device
  * looks up the array's device address with that device current: make it before any stream

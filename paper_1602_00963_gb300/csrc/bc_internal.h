@@ -42,12 +42,13 @@ struct DevMem {
 // Control block of one traversal workspace (device memory).
 constexpr int kPlainScanBlocks = 1024;  // CTAs of the per-source kernel the rescan supports
 struct PlainCtl {
-  unsigned long long qpack;  // packed queue/edge append counter
+  unsigned long long qpack[3];  // packed queue/edge append counter of level l (slot l % 3)
   unsigned long long ns;     // component size incl. removed leaves (Eq. 3's n)
   GridSync bar;
-  unsigned long long sigmax[2];  // largest sigma of level l (slot l & 1)
-  int level_ovf[2];          // some vertex of level l overflowed 2^64 (slot l & 1)
+  unsigned long long sigmax[3];  // largest sigma of level l where it was read (slot l % 3)
+  int level_ovf[3];          // some vertex of level l overflowed 2^64 (slot l % 3)
   int src_ovf;               // some vertex of the current source overflowed
+  int base;                  // first depth value above the call's sources
   int max_depth;
   long long ovf_sources;
   long long levels;
@@ -62,15 +63,16 @@ struct PlainCtl {
 // queue Q with level offsets Q_off, degree prefix CD, depth d, sigma, bitmaps, delta).
 struct PlainWS {
   int32_t n = 0;
-  int32_t *depth = nullptr;    // [n]  -1 = unvisited
+  int32_t base = 0;            // depth values of later calls start here; below: unvisited
+  int32_t *depth = nullptr;    // [n]
   int32_t *Q = nullptr;        // [n]  BFS queue, also the stack of Alg. 1
   int32_t *CD = nullptr;       // [n]  exclusive prefix of degrees in Q order
   int32_t *lvl_off = nullptr;  // [n+2] Q offset of each level
   int32_t *lvl_eoff = nullptr; // [n+2] CD value at each level start
   unsigned long long *sig = nullptr;  // [n] sigma mod 2^64
   uint32_t *ovf = nullptr;     // [nw] overflow bits
-  uint32_t *vis = nullptr;     // [nw] visited-before-this-level bits
-  uint32_t *front = nullptr;   // [nw] frontier bits (bottom-up)
+  uint32_t *vis = nullptr;     // [nw] bits of the vertices reached two levels ago or earlier
+  uint32_t *front = nullptr;   // [nw] bits of a level (two more such bitmaps lie in r)
   unsigned long long *acc = nullptr;  // [2n] successor sums of Alg. 5 (64.64 fixed point)
   double *r = nullptr;         // [n] (1 + delta + omega) / sigma
   double *xm = nullptr;        // [n] extended-range sigma: mantissa
@@ -171,8 +173,10 @@ struct PlainArgs {
 bc_status plain_ensure(Ctx *ctx, PlainWS *ws, int32_t n);
 void plain_free(Ctx *ctx, PlainWS *ws);
 bc_status plain_run(Ctx *ctx, PlainWS *ws, const PlainArgs &a, cudaStream_t st, bc_stats *acc);
-bc_status plain_run_view(const PlainWS &ws, const PlainArgs &a, int num_sms, uint64_t limit_ns,
+bc_status plain_run_view(const PlainWS &ws, const PlainArgs &a, int ctas, uint64_t limit_ns,
                          cudaStream_t st, int *dev_err);
+bc_status plain_launch_solo(const PlainWS &ws, const PlainArgs &a, int teams, size_t stride, int *bad,
+                            cudaStream_t st);
 
 // ---- per-source path on small graphs: one CTA per source (bc_cta.cu)
 constexpr int32_t kCtaMaxN = 65536;        // default for the per-source path up to this size

@@ -11,7 +11,7 @@
 //
 // Limits and rules:
 //   * n <= BC_NOALLOC_MAX_N; larger graphs are rejected with BC_EINVAL, and so are an odd
-//     nnz and any source id outside [0, n) (checked on the device before the traversal;
+//     nnz and any source id outside [0, n) (checked on the device before its traversal;
 //     the CSR itself is not validated).
 //   * The scratch (about 4.2 MB) is part of the library image: every GPU on which the
 //     library is loaded holds it until the process exits.
@@ -25,8 +25,9 @@
 //   * The first call on a device looks up the array's device address
 //     (cudaGetSymbolAddress) with that device current; make that first call before any
 //     stream capture.
-//   * A call waits for its own work: it synchronises the given stream (after the source
-//     check and after the traversal) before it returns.
+//   * A call waits for its own work: it synchronises the given stream (after the traversal; on
+//     larger graphs also after the source check) before it returns.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -36,27 +37,56 @@ namespace bcl {
 namespace {
 
 constexpr int kMaxN = BC_NOALLOC_MAX_N;
-constexpr size_t kN2 = (size_t)kMaxN + 2;
-constexpr size_t kNW = (size_t)kMaxN / 32 + 1;
-
 constexpr size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// byte offsets of the workspace arrays inside the scratch
-constexpr size_t o_depth = 0;
-constexpr size_t o_Q = o_depth + al256(kN2 * 4);
-constexpr size_t o_CD = o_Q + al256(kN2 * 4);
-constexpr size_t o_loff = o_CD + al256(kN2 * 4);
-constexpr size_t o_leoff = o_loff + al256(kN2 * 4);
-constexpr size_t o_sig = o_leoff + al256(kN2 * 4);
-constexpr size_t o_acc = o_sig + al256(kN2 * 8);
-constexpr size_t o_r = o_acc + al256(kN2 * 16);
-constexpr size_t o_xm = o_r + al256(kN2 * 8);
-constexpr size_t o_xe = o_xm + al256(kN2 * 8);
-constexpr size_t o_ovf = o_xe + al256(kN2 * 4);
-constexpr size_t o_vis = o_ovf + al256(kNW * 4);
-constexpr size_t o_front = o_vis + al256(kNW * 4);
-constexpr size_t o_ctl = o_front + al256(kNW * 4);
-constexpr size_t o_chk = o_ctl + al256(sizeof(PlainCtl));  // source-range check word
+// byte offsets of a workspace's arrays for n vertices (at the start of the scratch, or of a team's
+// slice of it)
+struct Layout {
+  size_t depth, Q, CD, loff, leoff, sig, acc, r, xm, xe, ovf, vis, front, ctl, bc, total;
+  constexpr explicit Layout(size_t n, bool with_bc)
+      : depth(0), Q(0), CD(0), loff(0), leoff(0), sig(0), acc(0), r(0), xm(0), xe(0), ovf(0), vis(0), front(0),
+        ctl(0), bc(0), total(0) {
+    const size_t N = n + 2, NW = n / 32 + 1;
+    Q = depth + al256(N * 4);
+    CD = Q + al256(N * 4);
+    loff = CD + al256(N * 4);
+    leoff = loff + al256(N * 4);
+    sig = leoff + al256(N * 4);
+    acc = sig + al256(N * 8);
+    r = acc + al256(N * 16);
+    xm = r + al256(N * 8);
+    xe = xm + al256(N * 8);
+    ovf = xe + al256(N * 4);
+    vis = ovf + al256(NW * 4);
+    front = vis + al256(NW * 4);
+    ctl = front + al256(NW * 4);
+    bc = ctl + al256(sizeof(PlainCtl));
+    total = bc + (with_bc ? al256(n * 8) : 0);
+  }
+  PlainWS at(unsigned char *base, int n) const {
+    PlainWS ws;
+    ws.n = n;
+    ws.depth = (int32_t *)(base + depth);
+    ws.Q = (int32_t *)(base + Q);
+    ws.CD = (int32_t *)(base + CD);
+    ws.lvl_off = (int32_t *)(base + loff);
+    ws.lvl_eoff = (int32_t *)(base + leoff);
+    ws.sig = (unsigned long long *)(base + sig);
+    ws.acc = (unsigned long long *)(base + acc);
+    ws.r = (double *)(base + r);
+    ws.xm = (double *)(base + xm);
+    ws.xe = (int32_t *)(base + xe);
+    ws.ovf = (uint32_t *)(base + ovf);
+    ws.vis = (uint32_t *)(base + vis);
+    ws.front = (uint32_t *)(base + front);
+    ws.ctl = (PlainCtl *)(base + ctl);
+    return ws;
+  }
+};
+constexpr Layout kFull(kMaxN, false);
+constexpr size_t o_depth = kFull.depth, o_sig = kFull.sig, o_acc = kFull.acc, o_xe = kFull.xe, o_ovf = kFull.ovf,
+                 o_vis = kFull.vis, o_front = kFull.front, o_ctl = kFull.ctl;
+constexpr size_t o_chk = kFull.total;  // source-range check word
 constexpr size_t kScratchBytes = o_chk + 256;
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
@@ -98,6 +128,18 @@ __global__ void k_noalloc_check(const int32_t *src, int32_t k, int32_t n, unsign
     if (src[i] < 0 || src[i] >= n) atomicOr((int *)(base + o_chk), 1);
 }
 
+// bc_out[v] = the teams' partials in team order, unless the check word is set
+__global__ void k_noalloc_reduce(const unsigned char *base, size_t stride, size_t o_bc, int teams, int n,
+                                 double *bc_out) {
+  if (*(const int *)(base + o_chk)) return;
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+    double sum = 0.0;
+#pragma unroll 4
+    for (int t = 0; t < teams; t++) sum += ((const double *)(base + stride * t + o_bc))[v];
+    bc_out[v] = sum;
+  }
+}
+
 std::mutex g_mu;
 unsigned char *g_addr[128];  // device address of g_scratch per device (set up once)
 
@@ -131,33 +173,6 @@ extern "C" bc_status bc_sources_noalloc(int32_t n, const int32_t *row_ptr, const
   cudaStream_t st = (cudaStream_t)cuda_stream;
   int sms = 0;
   BC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  k_noalloc_clear<<<sms * 4, 256, 0, st>>>(base, n);
-  BC_CUDA_TRY(cudaGetLastError());
-  if (k > 0) {
-    k_noalloc_check<<<sms, 256, 0, st>>>(src, k, n, base);
-    BC_CUDA_TRY(cudaGetLastError());
-    int bad = 0;
-    BC_CUDA_TRY(cudaMemcpyAsync(&bad, base + o_chk, sizeof(int), cudaMemcpyDeviceToHost, st));
-    BC_CUDA_TRY(cudaStreamSynchronize(st));
-    if (bad) return fail(BC_EINVAL, "bc_sources_noalloc: source id out of range [0, n)");
-  }
-  BC_CUDA_TRY(cudaMemsetAsync(bc_out, 0, (size_t)n * sizeof(double), st));
-  PlainWS ws;
-  ws.n = n;
-  ws.depth = (int32_t *)(base + o_depth);
-  ws.Q = (int32_t *)(base + o_Q);
-  ws.CD = (int32_t *)(base + o_CD);
-  ws.lvl_off = (int32_t *)(base + o_loff);
-  ws.lvl_eoff = (int32_t *)(base + o_leoff);
-  ws.sig = (unsigned long long *)(base + o_sig);
-  ws.acc = (unsigned long long *)(base + o_acc);
-  ws.r = (double *)(base + o_r);
-  ws.xm = (double *)(base + o_xm);
-  ws.xe = (int32_t *)(base + o_xe);
-  ws.ovf = (uint32_t *)(base + o_ovf);
-  ws.vis = (uint32_t *)(base + o_vis);
-  ws.front = (uint32_t *)(base + o_front);
-  ws.ctl = (PlainCtl *)(base + o_ctl);
   DeviceGraph g;
   g.n = n;
   g.nnz = nnz;
@@ -172,8 +187,46 @@ extern "C" bc_status bc_sources_noalloc(int32_t n, const int32_t *row_ptr, const
   a.max_degree = n;  // any degree is below n: a valid bound for the no-overflow test
   a.alpha = 0.5f;
   a.beta = 24.f;
+  // Small graphs: one CTA per source on a slice of the scratch each, as many as it holds; a level
+  // then ends in a CTA barrier instead of a grid barrier.  A source takes one CTA about 60 us
+  // + 1 ns per arc (R-MAT scale 10 / 12 / 14: 66 / 147 / 425 us), the whole GPU about 100 us and
+  // little more per arc (118 us at scale 12, 131 at 14), so the slices win while their rounds
+  // cost less.
+  const Layout lay((size_t)n, true);
+  const int teams = (int)std::min<size_t>(std::min<size_t>((size_t)std::max(k, 1), o_chk / lay.total), (size_t)sms);
+  if (k > 0 && teams > 0) {
+    const int64_t rounds = (k + teams - 1) / teams;
+    if (rounds * (60000 + nnz) <= (int64_t)k * 100000) {
+      BC_CUDA_TRY(cudaMemsetAsync(base + o_chk, 0, sizeof(int), st));
+      a.bc = (double *)(base + lay.bc);
+      const bc_status s = plain_launch_solo(lay.at(base, n), a, teams, lay.total, (int *)(base + o_chk), st);
+      if (s) return s;
+      k_noalloc_reduce<<<std::min((n + 255) / 256, sms), 256, 0, st>>>(base, lay.total, lay.bc, teams, n, bc_out);
+      BC_CUDA_TRY(cudaGetLastError());
+      int bad = 0;
+      BC_CUDA_TRY(cudaMemcpyAsync(&bad, base + o_chk, sizeof(int), cudaMemcpyDeviceToHost, st));
+      BC_CUDA_TRY(cudaStreamSynchronize(st));
+      if (bad) return fail(BC_EINVAL, "bc_sources_noalloc: source id out of range [0, n)");
+      return BC_OK;
+    }
+  }
+  k_noalloc_clear<<<sms * 4, 256, 0, st>>>(base, n);
+  BC_CUDA_TRY(cudaGetLastError());
+  if (k > 0) {
+    k_noalloc_check<<<sms, 256, 0, st>>>(src, k, n, base);
+    BC_CUDA_TRY(cudaGetLastError());
+    int bad = 0;
+    BC_CUDA_TRY(cudaMemcpyAsync(&bad, base + o_chk, sizeof(int), cudaMemcpyDeviceToHost, st));
+    BC_CUDA_TRY(cudaStreamSynchronize(st));
+    if (bad) return fail(BC_EINVAL, "bc_sources_noalloc: source id out of range [0, n)");
+  }
+  BC_CUDA_TRY(cudaMemsetAsync(bc_out, 0, (size_t)n * sizeof(double), st));
+  const PlainWS ws = kFull.at(base, n);
+  // the grid: barriers of fewer CTAs are cheaper, while the level's work fits them (R-MAT scale 12,
+  // per source: 118 us with 12 CTAs, 129 with all; scale 16: 162 with all, 278 with 8)
+  const int ctas = std::min(sms, nnz <= 150000 ? 12 : nnz <= 600000 ? 64 : sms);
   int derr = 0;
-  bc_status s = plain_run_view(ws, a, sms, 20ull * 1000 * 1000 * 1000, st, &derr);
+  const bc_status s = plain_run_view(ws, a, ctas, 20ull * 1000 * 1000 * 1000, st, &derr);
   if (s) return s;
   if (derr == BCD_TIMEOUT) return fail(BC_ETIMEDOUT, "bc_sources_noalloc: a grid barrier wait passed its limit");
   if (derr) return fail(BC_ECUDA, "bc_sources_noalloc: device error " + std::to_string(derr));

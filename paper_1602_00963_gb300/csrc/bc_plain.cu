@@ -11,13 +11,17 @@
 //     reuses it (the scan / search reuse of Sec. 3.1).  A warp keeps a window of 128
 //     CD entries in shared memory and has four 32-edge steps in flight at once.
 //   * Alg. 3 tests d[w] and adds sigma in one parallel loop, which can drop a term when
-//     a thread reads d[w] before another thread has set it.  Here the discovering
-//     compare-and-swap returns the previous depth, and a thread adds sigma exactly when
-//     that value is -1 (it discovered w) or the current level (w was discovered at this
-//     level), so every parent edge contributes once.
+//     a thread reads d[w] before another thread has set it.  Here an edge into a vertex not
+//     reached at an earlier level (a bitmap test) raises its depth with an atomic maximum,
+//     which tells the discoverer, and adds sigma in any case, so every parent edge contributes
+//     once.  Depth values carry a base that grows from source to source, so depths of earlier
+//     sources read as "not reached" and are not reset.
 //   * bottom-up levels (direction switch): each unvisited vertex sums sigma over all its
 //     neighbours in the frontier bitmap (all parents at level d-1, no early exit, so
 //     sigma stays exact).
+//   * the level bitmaps rotate: one is built, one is the frontier, one is cleared; the frontier is
+//     merged into the visited bitmap word by word beside the sweep, so a level needs one grid
+//     barrier and no pass over its vertices.
 //   * sigma is kept modulo 2^64 with a sticky overflow bit; vertices whose count
 //     overflows also get an extended-range value (double mantissa, int exponent).
 // Backward (dependency accumulation, Alg. 4 / Alg. 5, successor checking):
@@ -25,13 +29,15 @@
 //   d[v] = d[w] + 1 adds sigma[w] * r[v] = sigma[w] / sigma[v] * (1 + delta[v] + omega[v])
 //   to acc[w]; then delta[w] = acc[w] (updateDep), BC[w] += (omega[s] + 1) * delta[w]
 //   (Eq. 3 / Eq. 4) and r[w] = (1 + delta[w] + omega[w]) / sigma[w].  Each term lies in
-//   [0, n] and is added as a 128-bit fixed-point integer (64 fraction bits; warp-segmented
-//   sums, one pair of 64-bit integer atomics per segment): integer sums do not depend on
-//   the order of the additions, so the result repeats bit for bit from run to run.
+//   [0, n] and is added as a 128-bit fixed-point integer (64 fraction bits; per-lane and
+//   warp-segmented sums, one pair of 64-bit integer atomics per segment): integer sums do not
+//   depend on the order of the additions, so the result repeats bit for bit from run to run,
+//   and a level whose successors have few arcs sums over theirs instead.
 #include <climits>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "bc_internal.h"
 
@@ -43,7 +49,8 @@ constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int U = 4;             // 32-edge steps in flight per warp
 constexpr int WIN = 32 * U;      // owner window (queue entries) per warp
-constexpr unsigned kFound = 1u, kOvf = 2u;
+constexpr int kBaseMax = 1 << 30;  // depth values stay below (base + level)
+constexpr int kPushFactor = 2;     // backward: push from a level with at most half of the arcs
 
 struct WarpWin {
   int cd[WIN + 1];  // CD of window entries (INT_MAX past the range), then the next CD
@@ -67,7 +74,9 @@ struct PK {
   int leaf_term;
   int32_t *depth, *Q, *CD, *lvl_off, *lvl_eoff;
   unsigned long long *sig;
-  uint32_t *ovf, *vis, *front;
+  uint32_t *ovf, *vis;
+  uint32_t *lvb[3];         // bitmap of level l in lvb[l % 3]; 1 and 2 lie in r (idle in the forward sweep)
+  int32_t base;             // depth values of the first source start here; below: not reached
   unsigned long long *acc;  // [2n]: per vertex the low and high word of a 64.64 fixed-point sum
   double *r, *xm;
   int32_t *xe;
@@ -80,12 +89,18 @@ struct PK {
   unsigned long long *trace;  // optional phase trace: (phase << 56 | level << 32, time) pairs
   int trace_cap;
   int no_cd_reuse;            // backward: rescan CD per level (ablation)
+  int *bad;                   // plain_solo: set for a source id outside [0, n)
 };
 
 // Grid barrier; with tracing on, CTA 0 stamps the time at which every CTA has finished
 // the phase (so consecutive stamps give each phase's duration, slowest CTA included).
+template <bool SOLO = false>
 __device__ __forceinline__ bool phase_sync(const PK &p, GridSync *gs, int phase, int level) {
-  bool ok = grid_sync(gs, p.limit_ns);
+  if (SOLO) {  // one CTA runs the source: nobody to wait for
+    __syncthreads();
+    return true;
+  }
+  const bool ok = grid_sync(gs, p.limit_ns);
   if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) {
     int i = p.ctl->trace_n++;
     if (i < p.trace_cap) {
@@ -153,7 +168,10 @@ __device__ __forceinline__ int warp_find_owner(const int32_t *CD, int lo, int hi
 
 // Warp-aggregated append of up to U flagged vertices per lane to Q (and their degree
 // prefix to CD) with one packed atomicAdd per warp.
-__device__ __forceinline__ void warp_append_u(const PK &p, const int (&w)[U], const bool (&isnew)[U]) {
+// (ctr: the level's packed counter; its entries start at queue position q1, edge offset E1).
+// The vertices' bits in the level's bitmap are set here too.
+__device__ __forceinline__ void warp_append_u(const PK &p, const int (&w)[U], const bool (&isnew)[U],
+                                              unsigned long long *ctr, int q1, int E1, uint32_t *lvb) {
   int cnt = 0, dsum = 0;
   int dg[U];
 #pragma unroll
@@ -167,13 +185,14 @@ __device__ __forceinline__ void warp_append_u(const PK &p, const int (&w)[U], co
   int cpre = warp_excl_scan(cnt, &ctot);
   int dpre = warp_excl_scan(dsum, &dtot);
   unsigned long long base = 0;
-  if (lane_id() == 0) base = atomicAdd(&p.ctl->qpack, pack_qe((unsigned)ctot, (unsigned)dtot));
+  if (lane_id() == 0) base = atomicAdd(ctr, pack_qe((unsigned)ctot, (unsigned)dtot));
   base = __shfl_sync(BC_FULL, base, 0);
-  int pos = (int)(base >> 32) + cpre;
-  int eo = (int)(base & 0xffffffffull) + dpre;
+  int pos = q1 + (int)(base >> 32) + cpre;
+  int eo = E1 + (int)(base & 0xffffffffull) + dpre;
 #pragma unroll
   for (int k = 0; k < U; k++) {
     if (isnew[k]) {
+      set_bit_atomic(lvb, w[k]);
       p.Q[pos] = w[k];
       p.CD[pos] = eo;
       pos++;
@@ -182,7 +201,9 @@ __device__ __forceinline__ void warp_append_u(const PK &p, const int (&w)[U], co
   }
 }
 
-template <bool EXT, bool BWD>
+// What a window holds per entry besides its vertex: nothing (MODE 0), sigma (1; EXT: as m 2^e), or
+// r and its exponent (2).
+template <int MODE, bool EXT = false>
 __device__ __forceinline__ void fill_window(const PK &p, WarpWin &W, int base, int q1, int E1) {
   const int lane = lane_id();
   int vv[U], cc[U];
@@ -199,7 +220,11 @@ __device__ __forceinline__ void fill_window(const PK &p, WarpWin &W, int base, i
     W.cd[j] = cc[k];
     W.v[j] = vv[k];
     W.bias[j] = vv[k] >= 0 ? p.rp[vv[k]] - cc[k] : 0;
-    if (BWD) {
+    if (MODE == 2) {
+      W.sg[j] = vv[k] >= 0 ? p.r[vv[k]] : 0.0;
+      if (EXT) W.ex[j] = vv[k] >= 0 ? p.xe[vv[k]] : 0;
+    }
+    if (MODE == 1) {
       if (EXT) {
         const XS x = vv[k] >= 0 ? get_xs(p, vv[k]) : XS{0.0, 0};
         W.ex[j] = x.e;
@@ -223,7 +248,7 @@ __device__ __forceinline__ int win_owner(const WarpWin &W, int e) {
 
 // Iterate the warp's slice of the edge range [E0, E1) of queue range [q0, q1), U x 32
 // edges at a time.  body(e0, ee) is called once per window with the window filled.
-template <bool EXT, bool BWD, typename F>
+template <int MODE, bool EXT = false, typename F>
 __device__ __forceinline__ void edge_windows(const PK &p, WarpWin &W, int q0, int q1, int E0,
                                              int E1, int gwarp, int nwarps, F &&body) {
   long long E = (long long)E1 - E0;
@@ -236,7 +261,7 @@ __device__ __forceinline__ void edge_windows(const PK &p, WarpWin &W, int q0, in
   const int ee = (int)min(ebl + per, (long long)E1);
   int base = warp_find_owner(p.CD, q0, q1, eb);
   for (int e0 = eb; e0 < ee; e0 += WIN) {
-    fill_window<EXT, BWD>(p, W, base, q1, E1);
+    fill_window<MODE, EXT>(p, W, base, q1, E1);
     body(e0, ee);
     // next window starts at the owner of edge e0 + WIN
     int jl = win_owner(W, e0 + WIN - 1);
@@ -246,10 +271,27 @@ __device__ __forceinline__ void edge_windows(const PK &p, WarpWin &W, int q0, in
   }
 }
 
-__device__ void expand_topdown(const PK &p, WarpWin &W, int level, int q0, int q1, int E0,
-                               int E1, int gwarp, int nwarps, bool fast) {
+// The level in progress: its number and depth value, its slots and where its entries start.
+struct Lvl {
+  int level, dv;            // dv = base + level
+  int q1, E1;               // queue position and edge offset of its first entry
+  unsigned long long *ctr;  // packed append counter
+  int *ovf;                 // set when a vertex of the level passes 2^64
+  bool povf;                // vertices of earlier levels may have
+  uint32_t *cur;            // bitmap of the level (being built)
+  const uint32_t *front;    // bitmap of the level before
+};
+
+// Reached before this level: vis holds the levels up to level - 2, and is being merged with the
+// level before meanwhile.
+__device__ __forceinline__ bool reached_before(const PK &p, const Lvl &L, int v) {
+  return test_bit(p.vis, v) || test_bit(L.front, v);
+}
+
+__device__ void expand_topdown(const PK &p, WarpWin &W, const Lvl &L, int q0, int E0, int gwarp, int nwarps,
+                               bool fast) {
   const int lane = lane_id();
-  edge_windows<false, false>(p, W, q0, q1, E0, E1, gwarp, nwarps, [&](int e0, int ee) {
+  edge_windows<0>(p, W, q0, L.q1, E0, L.E1, gwarp, nwarps, [&](int e0, int ee) {
     int w[U], v[U];
     bool isnew[U], dag[U];
 #pragma unroll
@@ -263,10 +305,10 @@ __device__ void expand_topdown(const PK &p, WarpWin &W, int level, int q0, int q
     for (int k = 0; k < U; k++) {
       isnew[k] = false;
       dag[k] = false;
-      if (w[k] >= 0 && !test_bit(p.vis, w[k])) {
-        int old = atomicCAS(p.depth + w[k], -1, level);
-        isnew[k] = old < 0;
-        dag[k] = isnew[k] || old == level;
+      if (w[k] >= 0 && !reached_before(p, L, w[k])) {
+        int old = atomicMax(p.depth + w[k], L.dv);
+        isnew[k] = old < L.dv;
+        dag[k] = true;  // discovered here or by another parent at this level
       }
     }
 #pragma unroll
@@ -279,85 +321,120 @@ __device__ void expand_topdown(const PK &p, WarpWin &W, int level, int q0, int q
           unsigned long long old = atomicAdd(p.sig + w[k], sv);
           if (old + sv < old || test_bit(p.ovf, v[k])) {
             set_bit_atomic(p.ovf, w[k]);
-            p.ctl->level_ovf[level & 1] = 1;
+            *L.ovf = 1;
             p.ctl->src_ovf = 1;
           }
         }
       }
     }
-    warp_append_u(p, w, isnew);
+    warp_append_u(p, w, isnew, L.ctr, L.q1, L.E1, L.cur);
   });
 }
 
-__device__ void sweep_bottomup(const PK &p, int level, int gwarp, int nwarps,
-                               unsigned long long (*s_sig)[32], unsigned (*s_flag)[32]) {
+// s += v; ov: a carry out of bit 63, or v had passed 2^64 itself.
+__device__ __forceinline__ void sum_carry(unsigned long long &s, bool &ov, unsigned long long v, bool o) {
+  const unsigned long long t = s + v;
+  ov = ov || t < s || o;
+  s = t;
+}
+
+// Bottom-up level: 32 consecutive vertices per warp, those not reached yet sum sigma over their
+// neighbours in the frontier (all of them, no early exit).  A lane takes a row of up to
+// kBuLane arcs, four in flight; the warp takes larger rows together, one after another, and
+// reduces by shuffles.  Sums stay in registers: 64-bit additions to shared memory are
+// compare-and-swap loops, which the arcs of one vertex, next to each other in a step, repeated up
+// to 32 times (R-MAT scale 20: 363 us for a level-3 sweep with them).
+constexpr int kBuLane = 32;
+__device__ void sweep_bottomup(const PK &p, const Lvl &L, int gwarp, int nwarps) {
   const int lane = lane_id();
-  const int wl = threadIdx.x >> 5;
   for (int g = gwarp; g * 32 < p.n; g += nwarps) {
-    int u = g * 32 + lane;
-    bool act = u < p.n && !test_bit(p.vis, u);
+    const uint32_t seen = p.vis[g] | L.front[g];
+    if (seen == BC_FULL) continue;
+    const int u = g * 32 + lane;
     int st = 0, c = 0;
-    if (act) {
+    if (u < p.n && !((seen >> lane) & 1u)) {
       st = p.rp[u];
       c = p.rp[u + 1] - st;
     }
-    int tot;
-    int ex = warp_excl_scan(c, &tot);
-    if (tot == 0) continue;
-    s_sig[wl][lane] = 0ull;
-    s_flag[wl][lane] = 0u;
-    __syncwarp();
-    int bias = st - ex;
-    for (int e0 = 0; e0 < tot; e0 += WIN) {
-      int pn[U], jj[U];
+    unsigned long long sum = 0ull;
+    bool ov = false, found = false;
+    if (c <= kBuLane) {
+      for (int e = 0; e < c; e += U) {
+        int pn[U];
+        bool fr[U];
+        unsigned long long sv[U];
 #pragma unroll
-      for (int k = 0; k < U; k++) {
-        int my = e0 + lane + 32 * k;
-        jj[k] = warp_owner(ex, my);
-        int b = __shfl_sync(BC_FULL, bias, jj[k]);
-        pn[k] = my < tot ? p.ci[my + b] : -1;
-      }
-      bool fr[U];
+        for (int k = 0; k < U; k++) pn[k] = e + k < c ? p.ci[st + e + k] : -1;
 #pragma unroll
-      for (int k = 0; k < U; k++) fr[k] = pn[k] >= 0 && test_bit(p.front, pn[k]);
+        for (int k = 0; k < U; k++) fr[k] = pn[k] >= 0 && test_bit(L.front, pn[k]);
 #pragma unroll
-      for (int k = 0; k < U; k++) {
-        if (fr[k]) {
-          unsigned long long sv = p.sig[pn[k]];
-          unsigned long long old = atomicAdd(&s_sig[wl][jj[k]], sv);
-          unsigned fl = kFound;
-          if (old + sv < old || test_bit(p.ovf, pn[k])) fl |= kOvf;
-          atomicOr(&s_flag[wl][jj[k]], fl);
+        for (int k = 0; k < U; k++) sv[k] = fr[k] ? p.sig[pn[k]] : 0ull;
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+          if (!fr[k]) continue;
+          found = true;
+          sum_carry(sum, ov, sv[k], L.povf && test_bit(p.ovf, pn[k]));
         }
       }
     }
     __syncwarp();
-    unsigned f = s_flag[wl][lane];
-    bool isnew = act && (f & kFound);
-    int wv[U] = {u};
-    bool nv[U] = {isnew};
-    if (isnew) {
-      p.depth[u] = level;
-      p.sig[u] = s_sig[wl][lane];
-      if (f & kOvf) {
+    unsigned big = __ballot_sync(BC_FULL, c > kBuLane);
+    while (big) {
+      const int j = __ffs(big) - 1;
+      big &= big - 1;
+      const int s0 = __shfl_sync(BC_FULL, st, j), cj = __shfl_sync(BC_FULL, c, j);
+      unsigned long long s = 0ull;
+      bool o = false, f = false;
+      for (int e = lane; e < cj; e += 32 * U) {
+        int pn[U];
+        bool fr[U];
+        unsigned long long sv[U];
+#pragma unroll
+        for (int k = 0; k < U; k++) pn[k] = e + 32 * k < cj ? p.ci[s0 + e + 32 * k] : -1;
+#pragma unroll
+        for (int k = 0; k < U; k++) fr[k] = pn[k] >= 0 && test_bit(L.front, pn[k]);
+#pragma unroll
+        for (int k = 0; k < U; k++) sv[k] = fr[k] ? p.sig[pn[k]] : 0ull;
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+          if (!fr[k]) continue;
+          f = true;
+          sum_carry(s, o, sv[k], L.povf && test_bit(p.ovf, pn[k]));
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) sum_carry(s, o, __shfl_xor_sync(BC_FULL, s, d), false);
+      const bool ao = __any_sync(BC_FULL, o), af = __any_sync(BC_FULL, f);
+      if (lane == j) {
+        sum = s;
+        ov = ao;
+        found = af;
+      }
+    }
+    if (found) {
+      p.depth[u] = L.dv;
+      p.sig[u] = sum;
+      if (ov) {
         set_bit_atomic(p.ovf, u);
-        p.ctl->level_ovf[level & 1] = 1;
+        *L.ovf = 1;
         p.ctl->src_ovf = 1;
       }
     }
-    warp_append_u(p, wv, nv);
-    __syncwarp();
+    int wv[U] = {u};
+    bool nv[U] = {found};
+    warp_append_u(p, wv, nv, L.ctr, L.q1, L.E1, L.cur);
   }
 }
 
-// Extended-range sigma of an overflowed vertex: sum over its parents (d = level-1).
-__device__ void ext_sigma(const PK &p, int w, int level) {
+// Extended-range sigma of an overflowed vertex: sum over its parents (depth value dp).
+__device__ void ext_sigma(const PK &p, int w, int dp) {
   XS a;
   a.m = 0.0;
   a.e = 0;
   for (int e = p.rp[w]; e < p.rp[w + 1]; e++) {
     int x = p.ci[e];
-    if (p.depth[x] == level - 1) xs_add(a, get_xs(p, x));
+    if (p.depth[x] == dp) xs_add(a, get_xs(p, x));
   }
   a = xs_norm(a);
   p.xm[w] = a.m;
@@ -383,64 +460,117 @@ __device__ __forceinline__ void fx_from(double t, unsigned long long &hi, unsign
   }
 }
 
+// acc[o] += (hi, lo): integer additions, so their order does not matter.
+__device__ __forceinline__ void acc_add(const PK &p, int o, unsigned hi, unsigned long long lo) {
+  if (!(hi | lo)) return;
+  unsigned long long *a = p.acc + 2 * (size_t)o;
+  const unsigned long long old = lo ? atomicAdd(a, lo) : 0ull;
+  const unsigned long long c = (lo && old + lo < old) ? 1ull : 0ull;  // the low word wrapped
+  if (hi + c) atomicAdd(a + 1, hi + c);
+}
+
+// Level d's sums over the arcs (w, v) of its own entries w (pull).  A lane takes four consecutive
+// arcs of a window and adds up the terms of one owner as it goes; where the owner changes
+// inside its four arcs it writes the finished sum out, and only its last owner's sum goes
+// through the warp-segmented reduction, so that runs once per 128 arcs and not at all where no
+// arc leads to a successor.  hi: a sum of one owner's terms stays below n < 2^31.
 template <bool EXT>
-__device__ void accumulate_level(const PK &p, WarpWin &W, int d, int q0, int q1, int E0, int E1,
+__device__ void accumulate_level(const PK &p, WarpWin &W, int dn, int q0, int q1, int E0, int E1,
                                  int gwarp, int nwarps) {
   const int lane = lane_id();
-  edge_windows<EXT, true>(p, W, q0, q1, E0, E1, gwarp, nwarps, [&](int e0, int ee) {
-    int own[U], nb[U], ew[U];
-    double sw[U];
+  edge_windows<1, EXT>(p, W, q0, q1, E0, E1, gwarp, nwarps, [&](int e0, int ee) {
+    const int e = e0 + U * lane;
+    int j = win_owner(W, min(e, ee - 1));
+    int ow[U], nb[U];
 #pragma unroll
     for (int k = 0; k < U; k++) {
-      int e = e0 + lane + 32 * k;
-      int j = win_owner(W, e);
-      bool valid = e < ee;
-      own[k] = valid ? W.v[j] : -1;
-      ew[k] = EXT ? W.ex[j] : 0;
-      sw[k] = W.sg[j];
-      nb[k] = valid ? p.ci[e + W.bias[j]] : -1;
+      while (j < WIN - 1 && W.cd[j + 1] <= e + k) j++;
+      ow[k] = j;
+      nb[k] = e + k < ee ? p.ci[e + k + W.bias[j]] : -1;
     }
     int dv[U];
 #pragma unroll
-    for (int k = 0; k < U; k++) dv[k] = nb[k] >= 0 ? p.depth[nb[k]] : -9;
+    for (int k = 0; k < U; k++) dv[k] = nb[k] >= 0 ? p.depth[nb[k]] : -1;
     double val[U];
+    bool any = false;
 #pragma unroll
     for (int k = 0; k < U; k++) {
       val[k] = 0.0;
-      if (dv[k] == d + 1) {
+      if (nb[k] >= 0 && dv[k] == dn) {
         val[k] = p.r[nb[k]];
-        if (EXT) val[k] = ldexp(val[k], ew[k] - p.xe[nb[k]]);
-        val[k] *= sw[k];  // sigma[w] / sigma[v] * (1 + delta[v] + omega[v])
+        if (EXT) val[k] = ldexp(val[k], W.ex[ow[k]] - p.xe[nb[k]]);
+        val[k] *= W.sg[ow[k]];  // sigma[w] / sigma[v] * (1 + delta[v] + omega[v])
+        any = true;
       }
     }
+    if (!__any_sync(BC_FULL, any)) return;
+    unsigned hi = 0u;
+    unsigned long long lo = 0ull;
 #pragma unroll
     for (int k = 0; k < U; k++) {
-      unsigned long long hi, lo;
-      fx_from(val[k], hi, lo);
-      const int o = own[k];
+      if (k > 0 && ow[k] != ow[k - 1]) {
+        acc_add(p, W.v[ow[k - 1]], hi, lo);
+        hi = 0u;
+        lo = 0ull;
+      }
+      unsigned long long h, l;
+      fx_from(val[k], h, l);
+      lo += l;
+      hi += (unsigned)h + (lo < l ? 1u : 0u);
+    }
+    const int o = ow[U - 1];
 #pragma unroll
-      for (int s = 1; s < 32; s <<= 1) {
-        const unsigned long long yl = __shfl_down_sync(BC_FULL, lo, s);
-        const unsigned long long yh = __shfl_down_sync(BC_FULL, hi, s);
-        const int oo = __shfl_down_sync(BC_FULL, o, s);
-        if (lane + s < 32 && oo == o) {
-          const unsigned long long l2 = lo + yl;
-          hi += yh + (l2 < lo ? 1ull : 0ull);
-          lo = l2;
-        }
+    for (int s = 1; s < 32; s <<= 1) {
+      const unsigned long long yl = __shfl_down_sync(BC_FULL, lo, s);
+      const unsigned yh = __shfl_down_sync(BC_FULL, hi, s);
+      const int oo = __shfl_down_sync(BC_FULL, o, s);
+      if (lane + s < 32 && oo == o) {
+        lo += yl;
+        hi += yh + (lo < yl ? 1u : 0u);
       }
-      const int prev = __shfl_up_sync(BC_FULL, o, 1);
-      const bool head = (lane == 0) || (prev != o);
-      if (head && o >= 0 && (hi | lo)) {
-        unsigned long long *a = p.acc + 2 * (size_t)o;
-        const unsigned long long old = lo ? atomicAdd(a, lo) : 0ull;
-        const unsigned long long c = (lo && old + lo < old) ? 1ull : 0ull;  // the low word wrapped
-        if (hi + c) atomicAdd(a + 1, hi + c);
+    }
+    const int prev = __shfl_up_sync(BC_FULL, o, 1);
+    if (lane == 0 || prev != o) acc_add(p, W.v[o], hi, lo);
+  });
+}
+
+// The same sums over the arcs (v, w) of the next level's entries v (push): taken where that level
+// has far fewer arcs, as the last levels of a low-diameter graph do (R-MAT scale 20: the level
+// before the last walked 15 M arcs for the few thousand that lead on, 242 us).  The terms are
+// the same products, so the integer sums are too.
+template <bool EXT>
+__device__ void push_level(const PK &p, WarpWin &W, int dd, int q0, int q1, int E0, int E1, int gwarp, int nwarps) {
+  const int lane = lane_id();
+  edge_windows<2, EXT>(p, W, q0, q1, E0, E1, gwarp, nwarps, [&](int e0, int ee) {
+    int w[U], ow[U];
+#pragma unroll
+    for (int k = 0; k < U; k++) {
+      const int e = e0 + lane + 32 * k;
+      ow[k] = win_owner(W, e);
+      w[k] = e < ee ? p.ci[e + W.bias[ow[k]]] : -1;
+    }
+    int dv[U];
+#pragma unroll
+    for (int k = 0; k < U; k++) dv[k] = w[k] >= 0 ? p.depth[w[k]] : -1;
+#pragma unroll
+    for (int k = 0; k < U; k++) {
+      if (w[k] < 0 || dv[k] != dd) continue;
+      double val = W.sg[ow[k]];
+      if (EXT) {
+        const XS x = get_xs(p, w[k]);
+        val = ldexp(val, x.e - W.ex[ow[k]]) * x.m;
+      } else {
+        val *= (double)p.sig[w[k]];
       }
+      unsigned long long h, l;
+      fx_from(val, h, l);
+      acc_add(p, w[k], (unsigned)h, l);
     }
   });
 }
 
+// delta, BC and r of a level from its sums; sigma is not needed after it and is cleared for the
+// next source.
 template <bool EXT>
 __device__ void finalize_level(const PK &p, int q0, int q1, double ws, int gtid, int nthr) {
   for (int i = q0 + gtid; i < q1; i += nthr) {
@@ -463,6 +593,7 @@ __device__ void finalize_level(const PK &p, int q0, int q1, double ws, int gtid,
     }
     if (lo | hi) p.bc[w] += ws * delta;
     p.r[w] = (1.0 + delta + om) / sg;
+    p.sig[w] = 0ull;
   }
 }
 
@@ -534,52 +665,76 @@ __device__ bool rescan_level(const PK &p, GridSync *gs, int d, int q0, int q1, i
   return phase_sync(p, gs, 9, d);
 }
 
-__global__ void __launch_bounds__(kThreads, 1) plain_kernel(PK p) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned long long s_sig[kWarps][32];
-  __shared__ unsigned s_flag[kWarps][32];
-  __shared__ unsigned long long s_ns, s_max;
+// Start of a source: empty bitmaps but for the source's bit, its state, the control words.
+__device__ __forceinline__ void start_source(const PK &p, int s, int base, int gtid, int nthr) {
+  const int nw = (p.n + 31) / 32;
+  for (int i = gtid; i < nw; i += nthr) {
+    p.vis[i] = 0u;
+    p.ovf[i] = 0u;
+    p.lvb[0][i] = i == (s >> 5) ? 1u << (s & 31) : 0u;
+    p.lvb[1][i] = 0u;
+    p.lvb[2][i] = 0u;
+  }
+  if (gtid == 0) {
+    PlainCtl *ctl = p.ctl;
+    const int ds = p.rp[s + 1] - p.rp[s];
+    p.depth[s] = base;
+    p.sig[s] = 1ull;
+    p.Q[0] = s;
+    p.CD[0] = 0;
+    p.lvl_off[0] = 0;
+    p.lvl_off[1] = 1;
+    p.lvl_eoff[0] = 0;
+    p.lvl_eoff[1] = ds;
+    ctl->ns = 0ull;
+    ctl->src_ovf = 0;
+    for (int k = 0; k < 3; k++) {
+      ctl->qpack[k] = 0ull;
+      ctl->level_ovf[k] = 0;
+      ctl->sigmax[k] = 0ull;
+    }
+  }
+}
+
+// One grid barrier per level of the forward sweep (a second one only where a level passed 2^64 or
+// its largest sigma has to be known), two per level of the backward sweep.
+// SOLO: the CTA runs every team-th source of the list on a workspace of its own.
+template <bool SOLO>
+__device__ __forceinline__ void plain_body(const PK &p, unsigned char *smem) {
+  __shared__ unsigned long long s_red;
   WarpWin &W = ((WarpWin *)smem)[threadIdx.x >> 5];
-  const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nthr = gridDim.x * blockDim.x;
+  const int gtid = SOLO ? threadIdx.x : blockIdx.x * blockDim.x + threadIdx.x;
+  const int nthr = SOLO ? blockDim.x : gridDim.x * blockDim.x;
   const int gwarp = gtid >> 5;
   const int nwarps = nthr >> 5;
+  const int nw = (p.n + 31) / 32;
   PlainCtl *ctl = p.ctl;
   GridSync *gs = &ctl->bar;
   const bool sssp = p.out_depth != nullptr;
+  int base = p.base;
 
-  for (int si = 0; si < p.nsrc; ++si) {
+  for (int si = SOLO ? blockIdx.x : 0; si < p.nsrc; si += SOLO ? gridDim.x : 1) {
     const int s = p.src[si];
-    if (gtid == 0) {
-      int ds = p.rp[s + 1] - p.rp[s];
-      p.depth[s] = 0;
-      p.sig[s] = 1ull;
-      p.Q[0] = s;
-      p.CD[0] = 0;
-      p.lvl_off[0] = 0;
-      p.lvl_off[1] = 1;
-      p.lvl_eoff[0] = 0;
-      p.lvl_eoff[1] = ds;
-      ctl->qpack = pack_qe(1u, (unsigned)ds);
-      ctl->ns = 1ull + (p.omega ? (unsigned long long)p.omega[s] : 0ull);
-      ctl->src_ovf = 0;
-      ctl->level_ovf[0] = 0;
-      ctl->level_ovf[1] = 0;
-      ctl->sigmax[0] = 1ull;
-      ctl->sigmax[1] = 0ull;
-      set_bit_atomic(p.vis, s);
-      set_bit_atomic(p.front, s);
+    if (SOLO && (s < 0 || s >= p.n)) {
+      *p.bad = 1;
+      continue;
     }
-    if (!phase_sync(p, gs, 0, 0)) return;
+    if (base > kBaseMax - p.n) {  // depth values near their end: forget all sources before
+      for (int v = gtid; v < p.n; v += nthr) p.depth[v] = -1;
+      base = 0;
+      if (!phase_sync<SOLO>(p, gs, 0, 0)) return;
+    }
+    start_source(p, s, base, gtid, nthr);
+    if (!phase_sync<SOLO>(p, gs, 0, 0)) return;
 
     // ---------------------------------------------------------------- forward
     int level = 1;
     bool bu = false;
+    int q0 = 0, q1 = 1, E0 = 0, E1 = p.rp[s + 1] - p.rp[s];
+    double smax = 1.0;  // no sigma of the level before is larger (while none passed 2^64)
     while (true) {
-      const int q0 = p.lvl_off[level - 1], q1 = p.lvl_off[level];
       const int nf = q1 - q0;
       if (nf == 0) break;
-      const int E0 = p.lvl_eoff[level - 1], E1 = p.lvl_eoff[level];
       const double mf = (double)(E1 - E0);
       const double mu = (double)(p.nnz - E1);
       if (!bu) {
@@ -587,114 +742,194 @@ __global__ void __launch_bounds__(kThreads, 1) plain_kernel(PK p) {
       } else {
         if ((double)nf * (double)p.beta < (double)p.n && mf < (double)p.alpha * mu) bu = false;
       }
-      if (bu) {
-        sweep_bottomup(p, level, gwarp, nwarps, s_sig, s_flag);
-      } else {
-        // no 64-bit carry is possible this level if max sigma * max degree < 2^64
-        const bool fast = *(volatile int *)&ctl->src_ovf == 0 &&
-                          (double)*(volatile unsigned long long *)&ctl->sigmax[(level - 1) & 1] *
-                                  (double)p.max_degree < 1.8e19;
-        expand_topdown(p, W, level, q0, q1, E0, E1, gwarp, nwarps, fast);
-      }
-      if (!phase_sync(p, gs, bu ? 2 : 1, level)) return;
-
-      // post: level offsets, bitmaps, component size, level max sigma, extended sigma
-      const unsigned long long pk = *(volatile unsigned long long *)&ctl->qpack;
-      const int q2 = (int)(pk >> 32);
-      const bool lvl_ovf = *(volatile int *)&ctl->level_ovf[level & 1] != 0;
-      if (threadIdx.x == 0) {
-        s_ns = 0ull;
-        s_max = 0ull;
-      }
-      __syncthreads();
-      unsigned long long nsl = 0, mx = 0;
-      for (int i = q1 + gtid; i < q2; i += nthr) {
-        int w = p.Q[i];
-        set_bit_atomic(p.vis, w);
-        set_bit_atomic(p.front, w);
-        nsl += 1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull);
-        unsigned long long sw = p.sig[w];
-        mx = sw > mx ? sw : mx;
-        if (lvl_ovf && test_bit(p.ovf, w)) ext_sigma(p, w, level);
-      }
-      for (int i = q0 + gtid; i < q1; i += nthr) clear_bit_atomic(p.front, p.Q[i]);
-      if (nsl) atomicAdd(&s_ns, nsl);
-      if (mx) atomicMax(&s_max, mx);
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        if (s_ns) atomicAdd(&ctl->ns, s_ns);
-        if (s_max) atomicMax(&ctl->sigmax[level & 1], s_max);
+      Lvl L;
+      L.level = level;
+      L.dv = base + level;
+      L.q1 = q1;
+      L.E1 = E1;
+      L.ctr = &ctl->qpack[level % 3];
+      L.ovf = &ctl->level_ovf[level % 3];
+      L.povf = *(volatile int *)&ctl->src_ovf != 0;
+      L.cur = p.lvb[level % 3];
+      L.front = p.lvb[(level + 2) % 3];
+      uint32_t *old = p.lvb[(level + 1) % 3];  // level - 2: already in vis, the next level's
+      for (int i = gtid; i < nw; i += nthr) {
+        const uint32_t f = L.front[i];
+        if (f) p.vis[i] |= f;  // readers test vis and front, so either value serves them
+        if (old[i]) old[i] = 0u;
       }
       if (gtid == 0) {
-        p.lvl_off[level + 1] = q2;
-        p.lvl_eoff[level + 1] = (int)(pk & 0xffffffffull);
-        ctl->level_ovf[(level + 1) & 1] = 0;
-        ctl->sigmax[(level + 1) & 1] = 0ull;
+        ctl->qpack[(level + 1) % 3] = 0ull;
+        ctl->level_ovf[(level + 1) % 3] = 0;
+        ctl->sigmax[(level + 1) % 3] = 0ull;
       }
-      if (!phase_sync(p, gs, 3, level)) return;
+      if (bu) {
+        sweep_bottomup(p, L, gwarp, nwarps);
+      } else {
+        // no 64-bit carry is possible this level if max sigma * max degree < 2^64
+        const bool fast = !L.povf && smax * (double)p.max_degree < 1.8e19;
+        expand_topdown(p, W, L, q0, E0, gwarp, nwarps, fast);
+      }
+      if (!phase_sync<SOLO>(p, gs, bu ? 2 : 1, level)) return;
+
+      const unsigned long long pk = *(volatile unsigned long long *)L.ctr;
+      const int q2 = q1 + (int)(pk >> 32);
+      const bool lvl_ovf = *(volatile int *)L.ovf != 0;
+      // the level's largest sigma: bounded by the parents', read only where the bound would
+      // keep the next level from the carry-free additions
+      smax *= (double)p.max_degree;
+      const bool scan = smax * (double)p.max_degree >= 1.8e19 && *(volatile int *)&ctl->src_ovf == 0;
+      if ((lvl_ovf || scan) && q2 > q1) {
+        if (threadIdx.x == 0) s_red = 0ull;
+        __syncthreads();
+        unsigned long long mx = 0;
+        for (int i = q1 + gtid; i < q2; i += nthr) {
+          const int w = p.Q[i];
+          const unsigned long long sw = p.sig[w];
+          mx = sw > mx ? sw : mx;
+          if (lvl_ovf && test_bit(p.ovf, w)) ext_sigma(p, w, base + level - 1);
+        }
+        if (mx) atomicMax(&s_red, mx);
+        __syncthreads();
+        if (threadIdx.x == 0 && s_red) atomicMax(&ctl->sigmax[level % 3], s_red);
+        if (!phase_sync<SOLO>(p, gs, 3, level)) return;
+        smax = (double)*(volatile unsigned long long *)&ctl->sigmax[level % 3];
+      }
+      q0 = q1;
+      q1 = q2;
+      E0 = E1;
+      E1 += (int)(pk & 0xffffffffull);
+      if (gtid == 0) {
+        p.lvl_off[level + 1] = q1;
+        p.lvl_eoff[level + 1] = E1;
+      }
       level++;
     }
-    const int D = level - 2;                 // deepest non-empty level
-    const int qtot = p.lvl_off[level - 1];   // reached vertices
+    const int D = level - 2;   // deepest non-empty level
+    const int qtot = q1;       // reached vertices
 
     if (sssp) {
       for (int v = gtid; v < p.n; v += nthr) {
-        p.out_depth[v] = p.depth[v];
+        const int d = p.depth[v];
+        p.out_depth[v] = d >= base ? d - base : -1;
         p.out_sigma[v] = p.sig[v];
         p.out_ovf[v] = test_bit(p.ovf, v) ? 1 : 0;
+        p.sig[v] = 0ull;
       }
-      // every vertex is exported before any is reset below
-      if (!phase_sync(p, gs, 4, 0)) return;
     } else {
       // -------------------------------------------------------------- backward
       const bool ext = *(volatile int *)&ctl->src_ovf != 0;
       const double ws = p.omega ? (double)p.omega[s] + 1.0 : 1.0;
+      const bool leaf = p.leaf_term && p.omega && p.omega[s] > 0;
+      if (leaf && D >= 1) {  // n_s of Eq. 3
+        if (threadIdx.x == 0) s_red = 0ull;
+        __syncthreads();
+        unsigned long long part = 0;
+        for (int i = gtid; i < qtot; i += nthr) part += 1ull + (unsigned long long)p.omega[p.Q[i]];
+        if (part) atomicAdd(&s_red, part);
+        __syncthreads();
+        if (threadIdx.x == 0 && s_red) atomicAdd(&ctl->ns, s_red);
+      }
       if (D >= 1) {
+        // level offsets: written by one thread before a barrier each, or held in registers
+        int a0 = p.lvl_off[D], a1 = qtot, f0 = p.lvl_eoff[D], f1 = E1;
         if (ext)
-          finalize_level<true>(p, p.lvl_off[D], p.lvl_off[D + 1], ws, gtid, nthr);
+          finalize_level<true>(p, a0, a1, ws, gtid, nthr);
         else
-          finalize_level<false>(p, p.lvl_off[D], p.lvl_off[D + 1], ws, gtid, nthr);
-        if (!phase_sync(p, gs, 4, D)) return;
+          finalize_level<false>(p, a0, a1, ws, gtid, nthr);
+        if (!phase_sync<SOLO>(p, gs, 4, D)) return;
         for (int d = D - 1; d >= 1; --d) {
-          const int q0 = p.lvl_off[d], q1 = p.lvl_off[d + 1];
-          const int E0 = p.lvl_eoff[d], E1 = p.lvl_eoff[d + 1];
-          if (p.no_cd_reuse && !rescan_level(p, gs, d, q0, q1, E0)) return;
+          const int b0 = p.lvl_off[d], b1 = a0, g0 = p.lvl_eoff[d], g1 = f0;
+          if (!SOLO && p.no_cd_reuse && !rescan_level(p, gs, d, b0, b1, g0)) return;
+          // a pushed arc that leads back costs its own atomics, so push only from far fewer arcs
+          const bool push = !p.no_cd_reuse && (long long)(f1 - f0) * kPushFactor <= (long long)(g1 - g0);
+          if (push) {
+            if (ext)
+              push_level<true>(p, W, base + d, a0, a1, f0, f1, gwarp, nwarps);
+            else
+              push_level<false>(p, W, base + d, a0, a1, f0, f1, gwarp, nwarps);
+          } else {
+            if (ext)
+              accumulate_level<true>(p, W, base + d + 1, b0, b1, g0, g1, gwarp, nwarps);
+            else
+              accumulate_level<false>(p, W, base + d + 1, b0, b1, g0, g1, gwarp, nwarps);
+          }
+          if (!phase_sync<SOLO>(p, gs, 5, d)) return;
           if (ext)
-            accumulate_level<true>(p, W, d, q0, q1, E0, E1, gwarp, nwarps);
+            finalize_level<true>(p, b0, b1, ws, gtid, nthr);
           else
-            accumulate_level<false>(p, W, d, q0, q1, E0, E1, gwarp, nwarps);
-          if (!phase_sync(p, gs, 5, d)) return;
-          if (ext)
-            finalize_level<true>(p, q0, q1, ws, gtid, nthr);
-          else
-            finalize_level<false>(p, q0, q1, ws, gtid, nthr);
-          if (!phase_sync(p, gs, 6, d)) return;
+            finalize_level<false>(p, b0, b1, ws, gtid, nthr);
+          if (!phase_sync<SOLO>(p, gs, 6, d)) return;
+          a0 = b0;
+          a1 = b1;
+          f0 = g0;
+          f1 = g1;
         }
       }
-      if (gtid == 0 && p.leaf_term && p.omega && p.omega[s] > 0) {
-        double om = (double)p.omega[s];
-        double ns = (double)*(volatile unsigned long long *)&ctl->ns;
-        p.bc[s] += om * (2.0 * ns - om - 3.0);
+      if (gtid == 0) {
+        if (leaf) {
+          double om = (double)p.omega[s];
+          double ns = D >= 1 ? (double)*(volatile unsigned long long *)&ctl->ns : 1.0 + om;
+          p.bc[s] += om * (2.0 * ns - om - 3.0);
+        }
+        p.sig[s] = 0ull;
       }
     }
     if (gtid == 0) {
       if (*(volatile int *)&ctl->src_ovf) ctl->ovf_sources++;
       ctl->levels += level - 1;
       ctl->reached += qtot;
-      ctl->reached_arcs += p.lvl_eoff[level - 1];
+      ctl->reached_arcs += E1;
       if (D > ctl->max_depth) ctl->max_depth = D;
     }
-    // reset the state of the reached vertices for the next source
-    for (int i = gtid; i < qtot; i += nthr) {
-      int w = p.Q[i];
-      p.depth[w] = -1;
-      p.sig[w] = 0ull;
-      p.vis[w >> 5] = 0u;
-      p.front[w >> 5] = 0u;
-      p.ovf[w >> 5] = 0u;
-    }
-    if (!phase_sync(p, gs, 7, 0)) return;
+    base += D + 2;
+    // the next source's start overwrites what the phase after the last barrier may still read
+    if ((sssp || D == 0) && !phase_sync<SOLO>(p, gs, 7, 0)) return;
   }
+  if (gtid == 0) ctl->base = base;
+}
+
+__global__ void __launch_bounds__(kThreads, 1) plain_kernel(PK p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  plain_body<false>(p, smem);
+}
+
+// Team t's workspace lies t * stride bytes behind team 0's (p); it is cleared here.
+__global__ void __launch_bounds__(kThreads, 1) plain_solo(PK p, size_t stride) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ PK q;
+  if (threadIdx.x == 0) {
+    q = p;
+    const size_t o = stride * blockIdx.x;
+    auto move = [&](auto *&x) { x = (std::remove_reference_t<decltype(x)>)((char *)x + o); };
+    move(q.depth);
+    move(q.Q);
+    move(q.CD);
+    move(q.lvl_off);
+    move(q.lvl_eoff);
+    move(q.sig);
+    move(q.ovf);
+    move(q.vis);
+    for (int k = 0; k < 3; k++) move(q.lvb[k]);
+    move(q.acc);
+    move(q.r);
+    move(q.xm);
+    move(q.xe);
+    move(q.ctl);
+    move(q.bc);
+  }
+  __syncthreads();
+  for (int v = threadIdx.x; v < p.n; v += blockDim.x) {
+    q.depth[v] = -1;
+    q.sig[v] = 0ull;
+    q.acc[2 * v] = 0ull;
+    q.acc[2 * v + 1] = 0ull;
+    q.xe[v] = 0;
+    q.bc[v] = 0.0;
+  }
+  for (int i = threadIdx.x; i < (int)(sizeof(PlainCtl) / 4); i += blockDim.x) ((uint32_t *)q.ctl)[i] = 0u;
+  __syncthreads();
+  plain_body<true>(q, smem);
 }
 
 // The dynamic shared-memory size of plain_kernel is an attribute of the function on one
@@ -709,6 +944,8 @@ bc_status plain_setup(int *blocks_per_sm) {
   std::lock_guard<std::mutex> lk(g_setup_mu);
   if (!g_setup_done[dev]) {
     BC_CUDA_TRY(cudaFuncSetAttribute(plain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kSmemBytes));
+    BC_CUDA_TRY(cudaFuncSetAttribute(plain_solo, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSmemBytes));
     int b = 0;
     BC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, plain_kernel, kThreads, kSmemBytes));
@@ -745,6 +982,7 @@ static bc_status plain_reset(PlainWS *ws, cudaStream_t st) {
   BC_CUDA_TRY(cudaMemsetAsync(ws->acc, 0, N * 16, st));
   BC_CUDA_TRY(cudaMemsetAsync(ws->xe, 0, N * 4, st));
   BC_CUDA_TRY(cudaMemsetAsync(ws->ctl, 0, sizeof(PlainCtl), st));
+  ws->base = 0;
   return BC_OK;
 }
 
@@ -776,17 +1014,7 @@ bc_status plain_ensure(Ctx *ctx, PlainWS *ws, int32_t n) {
   return BC_OK;
 }
 
-// Launch the per-source kernel on a workspace whose arrays the caller has already laid
-// out (and cleared: depth -1; sigma, bitmaps, acc, exponents and the control block 0).
-// Allocates nothing and creates no events; waits for the kernel and reads its error word
-// into *dev_err.
-bc_status plain_run_view(const PlainWS &ws, const PlainArgs &a, int num_sms, uint64_t limit_ns,
-                         cudaStream_t st, int *dev_err) {
-  *dev_err = 0;
-  if (a.nsrc <= 0) return BC_OK;
-  int bps = 0;
-  bc_status s = plain_setup(&bps);
-  if (s) return s;
+static PK view_params(const PlainWS &ws, const PlainArgs &a, uint64_t limit_ns) {
   PK p;
   memset(&p, 0, sizeof(p));
   p.n = a.g->n;
@@ -807,23 +1035,60 @@ bc_status plain_run_view(const PlainWS &ws, const PlainArgs &a, int num_sms, uin
   p.sig = ws.sig;
   p.ovf = ws.ovf;
   p.vis = ws.vis;
-  p.front = ws.front;
+  p.lvb[0] = ws.front;
+  p.lvb[1] = (uint32_t *)ws.r;
+  p.lvb[2] = p.lvb[1] + (a.g->n + 31) / 32;
+  p.base = ws.base;
   p.acc = ws.acc;
   p.r = ws.r;
   p.xm = ws.xm;
   p.xe = ws.xe;
   p.ctl = ws.ctl;
+  p.out_depth = a.out_depth;
+  p.out_sigma = a.out_sigma;
+  p.out_ovf = a.out_ovf;
   p.alpha = a.alpha;
   p.beta = a.beta;
   p.limit_ns = limit_ns;
+  p.no_cd_reuse = a.no_cd_reuse ? 1 : 0;
+  return p;
+}
+
+// Launch the per-source kernel on a workspace whose arrays the caller has already laid
+// out (and cleared: depth -1; sigma, acc, exponents and the control block 0).
+// Allocates nothing and creates no events; waits for the kernel and reads its error word
+// into *dev_err.
+bc_status plain_run_view(const PlainWS &ws, const PlainArgs &a, int ctas, uint64_t limit_ns,
+                         cudaStream_t st, int *dev_err) {
+  *dev_err = 0;
+  if (a.nsrc <= 0) return BC_OK;
+  int bps = 0;
+  bc_status s = plain_setup(&bps);
+  if (s) return s;
+  PK p = view_params(ws, a, limit_ns);
   void *args[] = {&p};
-  cudaError_t le = cudaLaunchCooperativeKernel((void *)plain_kernel, dim3(num_sms * bps),
+  cudaError_t le = cudaLaunchCooperativeKernel((void *)plain_kernel, dim3(ctas * bps),
                                                dim3(kThreads), args, kSmemBytes, st);
   if (le != cudaSuccess) return cuda_fail(le, "cudaLaunchCooperativeKernel(plain_kernel)");
   int err = 0;
   BC_CUDA_TRY(cudaMemcpyAsync(&err, &ws.ctl->bar.err, sizeof(int), cudaMemcpyDeviceToHost, st));
   BC_CUDA_TRY(cudaStreamSynchronize(st));
   *dev_err = err;
+  return BC_OK;
+}
+
+// The same for `teams` CTAs that run different sources, each on a workspace of its own: team t's
+// lies t * stride bytes behind ws, with its BC partial (a.bc: team 0's).  Clears the workspaces;
+// sets *bad (device) for source ids outside [0, n), which are skipped.  Does not wait.
+bc_status plain_launch_solo(const PlainWS &ws, const PlainArgs &a, int teams, size_t stride, int *bad,
+                            cudaStream_t st) {
+  int bps = 0;
+  bc_status s = plain_setup(&bps);
+  if (s) return s;
+  PK p = view_params(ws, a, 0);
+  p.bad = bad;
+  plain_solo<<<teams, kThreads, kSmemBytes, st>>>(p, stride);
+  BC_CUDA_TRY(cudaGetLastError());
   return BC_OK;
 }
 
@@ -834,40 +1099,7 @@ bc_status plain_run(Ctx *ctx, PlainWS *ws, const PlainArgs &a, cudaStream_t st, 
     const bc_status s = plain_setup(&bps);
     if (s) return s;
   }
-  PK p;
-  p.n = a.g->n;
-  p.nnz = a.g->nnz;
-  p.max_degree = a.max_degree;
-  p.rp = a.g->rp;
-  p.ci = a.g->ci;
-  p.omega = a.omega;
-  p.src = a.src;
-  p.nsrc = a.nsrc;
-  p.bc = a.bc;
-  p.leaf_term = a.leaf_term ? 1 : 0;
-  p.depth = ws->depth;
-  p.Q = ws->Q;
-  p.CD = ws->CD;
-  p.lvl_off = ws->lvl_off;
-  p.lvl_eoff = ws->lvl_eoff;
-  p.sig = ws->sig;
-  p.ovf = ws->ovf;
-  p.vis = ws->vis;
-  p.front = ws->front;
-  p.acc = ws->acc;
-  p.r = ws->r;
-  p.xm = ws->xm;
-  p.xe = ws->xe;
-  p.ctl = ws->ctl;
-  p.out_depth = a.out_depth;
-  p.out_sigma = a.out_sigma;
-  p.out_ovf = a.out_ovf;
-  p.alpha = a.alpha;
-  p.beta = a.beta;
-  p.limit_ns = ctx->wait_limit_ns;
-  p.trace = nullptr;
-  p.trace_cap = 0;
-  p.no_cd_reuse = a.no_cd_reuse ? 1 : 0;
+  PK p = view_params(*ws, a, ctx->wait_limit_ns);
   if (a.no_cd_reuse && ctx->num_sms * bps > kPlainScanBlocks)
     return fail(BC_EINVAL, "BC_NO_CD_REUSE: more CTAs than the rescan supports");
   static const char *trace_file = getenv("BC_TRACE_FILE");
@@ -921,6 +1153,7 @@ bc_status plain_run(Ctx *ctx, PlainWS *ws, const PlainArgs &a, cudaStream_t st, 
       return fail(BC_ETIMEDOUT, "per-source kernel: a grid barrier wait passed its limit");
     return fail(BC_ECUDA, "per-source kernel reported device error " + std::to_string(h.bar.err));
   }
+  ws->base = h.base;
   if (acc) {
     acc->seconds += ms * 1e-3;
     acc->sources += a.nsrc;
