@@ -1100,8 +1100,8 @@ struct CtaPlan {
 // * 64 registers and 1024 threads per SM where rows beyond 64 arcs keep whole warps busy (R-MAT
 //   scale 12 all sources 3.3 against 4.1 with 128 registers and 512 threads; social graph above
 //   10.0 against 10.7), else 128 registers and 512 threads (G(9000, 36,000) all sources 9.0
-//   against 10.0), a lane then taking rows of up to 32 arcs instead of 16 (G(9000, 72,000):
-//   12.9 against 16.4).  From global memory 128 registers (64 spill in the sweeps: grid 1024^2
+//   against 10.0), a lane then taking rows of up to 32 arcs instead of 12 (G(9000, 72,000): 12.9,
+//   with 16 16.4, with 12 20.5; the social graph 9.6 with 12, 9.9 with 16, 11.1 with 32).  From global memory 128 registers (64 spill in the sweeps: grid 1024^2
 //   92 against 70); narrow graphs need no code for larger rows and run with 80 (59).
 // * Threads: an SM's threads over the states that fit it and have a source (one source on
 //   n = 1000: 85 us with 512, 95 with 128); from global memory 512 (social graph
@@ -1125,7 +1125,7 @@ static bc_status cta_plan(Ctx *ctx, int n, int max_degree, int units, bool tri, 
     pl->kernel = (const void *)k_cta_sources<true, false, 640, kNarrowDeg>;
   else
     pl->kernel = lb == 512 ? (const void *)k_cta_sources<true, false, 512, 32>
-                           : (const void *)k_cta_sources<true, false, 1024, 16>;
+                           : (const void *)k_cta_sources<true, false, 1024, 12>;
   pl->smem = sm ? cta_smem_bytes(n, cta_smem_q(n)) : sizeof(int32_t) * 2 * kRing;
   const int busy = std::min(per_sm, (units + ctx->num_sms - 1) / ctx->num_sms);  // CTAs per SM in use
   if (sm)
@@ -1144,7 +1144,7 @@ static bc_status cta_plan(Ctx *ctx, int n, int max_degree, int units, bool tri, 
     if (dev < 0 || dev >= 64 || !done[dev]) {
       for (const void *k : {(const void *)k_cta_sources<true, false, 640, kNarrowDeg>,
                             (const void *)k_cta_sources<true, false, 512, 32>,
-                            (const void *)k_cta_sources<true, false, 1024, 16>})
+                            (const void *)k_cta_sources<true, false, 1024, 12>})
         BC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtaSmemMax));
       if (dev >= 0 && dev < 64) done[dev] = true;
     }
