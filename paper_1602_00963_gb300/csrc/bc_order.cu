@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "bc_internal.h"
+#include "bc_scan.cuh"
 
 namespace bcl {
 
@@ -45,6 +46,23 @@ __global__ void k_lm_pack(const int32_t *depth, size_t total, uint8_t *out) {
   }
 }
 
+// flag[v] = 1 for a vertex with an edge, flag[n] = 0
+__global__ void k_lm_flags(int n, const int32_t *rp, int32_t *flag) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v <= n; v += (int64_t)gridDim.x * blockDim.x)
+    flag[v] = (v < n && rp[v + 1] > rp[v]) ? 1 : 0;
+}
+// pick[i]: a rank among the flagged vertices, replaced by the vertex (the last v with pos[v] <= rank)
+__global__ void k_lm_pick(int n, const int32_t *pos, int32_t *pick, int L) {
+  const int i = threadIdx.x;
+  if (i >= L) return;
+  int lo = 0, hi = n;
+  while (hi - lo > 1) {
+    const int mid = lo + (hi - lo) / 2;
+    if (pos[mid] <= pick[i]) lo = mid; else hi = mid;
+  }
+  pick[i] = lo;
+}
+
 // key[i * L + t] = distance of source i from landmark t
 __global__ void k_lm_gather(const uint8_t *d, int L, int n, const int32_t *src, int k, uint8_t *key) {
   const size_t total = (size_t)k * L;
@@ -57,19 +75,37 @@ __global__ void k_lm_gather(const uint8_t *d, int L, int n, const int32_t *src, 
 bc_status build_cache(Graph *g, const DeviceGraph *dg, int T, cudaStream_t st, TileWS **ws, OrderCache *oc) {
   Ctx *c = g->ctx;
   const int32_t n = dg->n;
-  std::vector<int32_t> rp((size_t)n + 1);
-  BC_CUDA_TRY(cudaMemcpyAsync(rp.data(), dg->rp, rp.size() * 4, cudaMemcpyDeviceToHost, st));
-  BC_CUDA_TRY(cudaStreamSynchronize(st));
-  std::vector<int32_t> pool;
-  for (int32_t v = 0; v < n; v++)
-    if (rp[v + 1] > rp[v]) pool.push_back(v);
   oc->rp = dg->rp;
   oc->L = 0;
-  if (pool.empty()) return BC_OK;
-  const int L = (int)std::min<size_t>(kLandmarks, pool.size());
-  std::vector<int64_t> idx = sample_distinct((int64_t)pool.size(), L, kLandmarkSeed);
+  // the landmarks: a seeded sample of the non-isolated vertices in increasing order, picked on the
+  // device by rank (flags, exclusive scan, one search per landmark)
+  const size_t n1 = (size_t)n + 1, b_arr = (n1 * 4 + 255) & ~(size_t)255;
+  char *tmp = nullptr;
+  cudaError_t ce = cudaMalloc(&tmp, 2 * b_arr + 256 + scan_scratch_bytes((int64_t)n1));
+  int32_t *flag = (int32_t *)tmp, *pos = (int32_t *)(tmp + b_arr), *pick = (int32_t *)(tmp + 2 * b_arr);
+  int32_t pool = 0;
+  if (ce == cudaSuccess) {
+    k_lm_flags<<<c->num_sms * 4, 256, 0, st>>>(n, dg->rp, flag);
+    ce = scan_exclusive_i32(flag, pos, (int64_t)n1, tmp + 2 * b_arr + 256, st);
+  }
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(&pool, pos + n, 4, cudaMemcpyDeviceToHost, st);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+  const int L = (int)std::min<int64_t>(kLandmarks, pool);
   std::vector<int32_t> lm((size_t)L);
-  for (int i = 0; i < L; i++) lm[i] = pool[(size_t)idx[i]];
+  if (ce == cudaSuccess && L > 0) {
+    std::vector<int64_t> idx = sample_distinct((int64_t)pool, L, kLandmarkSeed);
+    for (int i = 0; i < L; i++) lm[i] = (int32_t)idx[i];
+    ce = cudaMemcpyAsync(pick, lm.data(), (size_t)L * 4, cudaMemcpyHostToDevice, st);
+    k_lm_pick<<<1, 32, 0, st>>>(n, pos, pick, L);
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(lm.data(), pick, (size_t)L * 4, cudaMemcpyDeviceToHost, st);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+  }
+  if (tmp) cudaFree(tmp);
+  if (ce != cudaSuccess) {
+    oc->rp = nullptr;
+    return cuda_fail(ce, "source order: landmarks");
+  }
+  if (L == 0) return BC_OK;
   int32_t *d_lm = nullptr, *d_depth = nullptr;
   const size_t b_lm = (size_t)L * 4, b_depth = (size_t)L * n * 4, b_out = (size_t)L * n;
   bc_status s = c->mem.alloc((void **)&d_lm, b_lm);

@@ -50,6 +50,7 @@
 // kernel with bounded grid barriers (loop_mode 0), one launch per phase (1), and the
 // per-phase launches of kLevelsPerChunk levels captured once as a CUDA graph and
 // replayed until the level loop ends (2).
+#include <algorithm>
 #include <climits>
 #include <cstdio>
 #include <cstring>
@@ -105,10 +106,19 @@ struct TileCtl {
   unsigned long long ns[256];   // Eq. 3 component size per lane (leaf term)
 };
 
+// What the host reads of a finished tile (written by k_tile_end, one per tile of a batch).
+struct TileSum {
+  int err, lmax, ovf_sources, pad;
+  long long levels;
+  unsigned long long reached, reached_arcs;
+};
+constexpr int kTileBatch = 64;  // tiles launched before the host reads their sums
+
 }  // namespace
 
 struct TileWS {
   int n = 0, T = 0, G = 0;
+  int *stop = nullptr;  // set once a tile of a batch failed (then kTileBatch sums)
   int64_t capA = 0;
   bool ext_arrays = false;
   bool ext_sticky = false;  // this graph needed extended sigma before: start tiles in it
@@ -185,6 +195,7 @@ struct TK {
   int hub;        // degree from which a vertex is processed by whole CTAs / chunked
   int hub_chunk;  // edges of a hub per backward work item
   uint64_t limit_ns;
+  const int *stop;                // non-null: a tile before this one failed (nothing to do)
   int nreq;                       // > 0: lanes route BC to per-request buffers (serving)
   const uint8_t *lane_req;        // [T] request slot of each lane
   double *const *req_bc;          // [nreq] device BC buffers
@@ -1915,8 +1926,9 @@ __device__ void bwd_warp_item(const TK &p, int i, int h0, const uint32_t *Dn) {
   bwd_start_k<G, EXT>(p, k, o);
   const int e0 = p.rp[w] + c * p.hub_chunk, e1 = min(p.rp[w + 1], e0 + p.hub_chunk);
   // a pipeline over the 32-edge steps: neighbour ids two steps ahead, their masks one step
-  // ahead (in flight while a step's hits are summed), and the dense rows of the next step
-  // requested from L2 as soon as its masks are in
+  // ahead (in flight while a step's hits are summed).  A step's dense rows are requested from L2
+  // once, when the step begins: asking for the next step's as well doubled the requests (eight
+  // 32-line instructions a step at T = 128), 10.53 against 10.37 ms per tile of 128
   int vn = e0 + lane < e1 ? p.ci[e0 + lane] : -1;
   uint32_t bn[G];
 #pragma unroll
@@ -1940,16 +1952,6 @@ __device__ void bwd_warp_item(const TK &p, int i, int h0, const uint32_t *Dn) {
     bwd_hit_load<G, EXT>(p, h);
     if (h.hit && !h.sp) prefetch_row<G>(p.r + sidx<G>(h.v, 0, 0), h.bm);
     bwd_hits_add<G, EXT>(p, h, __ballot_sync(BC_FULL, h.sp), __ballot_sync(BC_FULL, h.hit && !h.sp), o);
-    if (vn >= 0) {  // the next step's dense rows
-      uint32_t m[G];
-      int nb = 0;
-#pragma unroll
-      for (int g = 0; g < G; g++) {
-        m[g] = bn[g] & o.mw[g];
-        nb += __popc(m[g]);
-      }
-      if (nb > kSparse) prefetch_row<G>(p.r + sidx<G>(vn, 0, 0), m);
-    }
   }
   if (nch == 1) {
     bwd_commit<G, EXT>(p, w, o);
@@ -2193,6 +2195,7 @@ __global__ void __launch_bounds__(TPB<G>::value, 1) tile_persistent(TK p, int fw
   const int nthr = gridDim.x * blockDim.x;
   const int gwarp = warp_rank(), nwarps = nthr >> 5;
   GridSync *gs = &p.ctl->bar;
+  if (p.stop && *p.stop) return;  // written by a kernel before this one
   sparse_acc_clear<G>();
   phase_init_vis<G>(p, gtid, nthr);
   if (!tsync(p, gs, 0, 0)) return;
@@ -2443,6 +2446,21 @@ __global__ void k_hub_chunks(const int32_t *hubs, int nh, const int32_t *rp, int
   }
 }
 
+// End of a tile launched without waiting: its sums to slot out, and the batch stopped if it failed.
+__global__ void k_tile_end(const TileCtl *c, int *stop, TileSum *out) {
+  if (*stop) return;
+  TileSum t;
+  t.err = c->bar.err;
+  t.lmax = c->lmax;
+  t.ovf_sources = t.pad = 0;
+  for (int g = 0; g < 8; g++) t.ovf_sources += __popc(c->ovf_lanes[g]);
+  t.levels = c->levels;
+  t.reached = c->reached;
+  t.reached_arcs = c->reached_arcs;
+  *out = t;
+  if (t.err) *stop = 1;
+}
+
 __global__ void k_wsrc(const int32_t *src, int nsrc, const int32_t *omega, float2 *wsrc, int T) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < T)
@@ -2495,7 +2513,7 @@ static void ws_release(Ctx *ctx, TileWS *ws, bool main, bool ext, bool A) {
   }
   if (main && ws->ctl) {
     void *ptrs[] = {ws->vis, ws->F, ws->ovf, ws->cand, ws->sig, ws->r, ws->Aoff, ws->Lbits, ws->HEoff,
-                    ws->C, ws->CPD, ws->CRP, ws->Ch, ws->ChP, ws->Fdone, ws->wsrc, ws->ctl};
+                    ws->C, ws->CPD, ws->CRP, ws->Ch, ws->ChP, ws->Fdone, ws->wsrc, ws->ctl, ws->stop};
     for (void *q : ptrs) cudaFree(q);
     ctx->mem.release(nullptr, ws->bytes_main);
     ws->vis = ws->F = ws->ovf = ws->cand = nullptr;
@@ -2505,6 +2523,7 @@ static void ws_release(Ctx *ctx, TileWS *ws, bool main, bool ext, bool A) {
     ws->Lbits = nullptr;
     ws->wsrc = nullptr;
     ws->ctl = nullptr;
+    ws->stop = nullptr;
     ws->bytes_main = 0;
   }
   if (ext && ws->ext_arrays) {
@@ -2586,6 +2605,7 @@ static bc_status ws_main(Ctx *ctx, TileWS *ws, int n, int T, cudaStream_t st) {
   TA(ws->Fdone, N * 4);
   TA(ws->wsrc, (size_t)T * 8);
   TA(ws->ctl, sizeof(TileCtl));
+  TA(ws->stop, 16 + kTileBatch * sizeof(TileSum));
   ws->n = n;
   ws->T = T;
   ws->G = G;
@@ -2814,17 +2834,22 @@ static bc_status capture_chunk(cudaStream_t st, cudaGraphExec_t *out, const KPtr
   return BC_OK;
 }
 
-// Run one tile (forward + backward) in loop mode `mode`; returns the device error code in
-// *derr and the number of kernel launches in *launches.
-static bc_status run_tile(Ctx *ctx, TileWS *ws, TK &p, int G, bool ext, int mode, bool fwd_only,
-                          cudaStream_t st, int *derr, int64_t *launches, int *lmax_out) {
+static bc_status tile_clear(TileWS *ws, int G, cudaStream_t st) {
   const size_t N = (size_t)ws->n, NG = N * G;
-  const KPtrs k = kptrs(G, ext);
-  bc_status s = BC_OK;
   BC_CUDA_TRY(cudaMemsetAsync(ws->F, 0, NG * 4 * 3, st));
   BC_CUDA_TRY(cudaMemsetAsync(ws->ovf, 0, NG * 4, st));
   BC_CUDA_TRY(cudaMemsetAsync(ws->ctl, 0, sizeof(TileCtl), st));
   BC_CUDA_TRY(cudaMemsetAsync(ws->Fdone, 0, N * 4, st));  // last-finisher counters (a failed tile may leave some set)
+  return BC_OK;
+}
+
+// Run one tile (forward + backward) in loop mode `mode`; returns the device error code in
+// *derr and the number of kernel launches in *launches.
+static bc_status run_tile(Ctx *ctx, TileWS *ws, TK &p, int G, bool ext, int mode, bool fwd_only,
+                          cudaStream_t st, int *derr, int64_t *launches, int *lmax_out) {
+  const KPtrs k = kptrs(G, ext);
+  bc_status s = tile_clear(ws, G, st);
+  if (s) return s;
   const int nsm = ctx->num_sms;
   const dim3 grid(nsm), block(k.tpb);
   *launches = 0;
@@ -2960,7 +2985,155 @@ bc_status tile_run(Ctx *ctx, Graph *g, TileWS **wsp, const TileArgs &a, cudaStre
   unsigned long long *trace_buf = nullptr;
   int64_t launches_total = 0, levels_total = 0, ovf_sources = 0, reached = 0, reached_arcs = 0;
   int maxd = 0;
-  for (int t0 = 0; t0 < a.nsrc && !s; t0 += a.T) {
+  // kernel parameters of the tile at sources [t0, t0 + nt)
+  auto params = [&](int t0, int nt) {
+    TK p;
+    memset(&p, 0, sizeof(p));
+    p.n = dg->n;
+    p.nnz = dg->nnz;
+    p.nsrc = nt;
+    p.rp = dg->rp;
+    p.ci = dg->ci;
+    p.omega = a.omega;
+    p.src = a.src + t0;
+    p.bc = a.bc;
+    p.leaf_term = a.omega != nullptr;
+    p.vis = ws->vis;
+    p.F = ws->F;
+    p.ovf = ws->ovf;
+    p.cand = ws->cand;
+    p.sig = ws->sig;
+    p.r = ws->r;
+    p.xm = ws->xm;
+    p.xe = ws->xe;
+    p.A = ws->A;
+    p.ACD = ws->ACD;
+    p.ARP = ws->ARP;
+    p.AM = ws->AM;
+    p.capA = ws->capA;
+    p.Aoff = ws->Aoff;
+    p.Lbits = ws->Lbits;
+    p.HE = ws->HE;
+    p.HEoff = ws->HEoff;
+    p.HEk = ws->HEk;
+    p.Hdone = ws->Hdone;
+    p.Hpart = ws->Hpart;
+    p.FPs = (unsigned long long *)ws->Hpart;
+    p.FPm = ws->FPm;
+    p.FPx = ws->FPx;
+    p.FPe = ws->FPe;
+    p.Fdone = ws->Fdone;
+    p.HPbu = ws->HPbu;
+    p.nhub_items = ws->nhub_items;
+    p.C = ws->C;
+    p.CPD = ws->CPD;
+    p.CRP = ws->CRP;
+    p.Ch = ws->Ch;
+    p.ChP = ws->ChP;
+    p.hubs = ws->hubs;
+    p.Lbu = ws->Lbu;
+    p.PDbu = ws->PDbu;
+    p.RPbu = ws->RPbu;
+    p.nhubs = ws->nhubs;
+    p.nbu = ws->nbu;
+    p.Ebu = ws->Ebu;
+    p.wsrc = ws->wsrc;
+    p.ctl = ws->ctl;
+    for (int gi = 0; gi < 8; gi++) {
+      uint32_t m = 0;
+      for (int b = 0; b < 32; b++)
+        if (gi * 32 + b >= nt) m |= 1u << b;
+      p.unused[gi] = m;
+    }
+    p.alpha = a.alpha;
+    p.beta = a.beta;
+    p.hub = hub;
+    p.hub_chunk = hub_chunk;
+    p.nreq = a.nreq;
+    p.lane_req = a.lane_req ? a.lane_req + t0 : nullptr;
+    p.req_bc = a.req_bc;
+    p.limit_ns = ctx->wait_limit_ns;
+    return p;
+  };
+  // Tiles of the persistent loop are launched up to kTileBatch in a row; the host waits once per
+  // batch, not after each tile (a wait, two copies and the launches behind them left the GPU idle
+  // for about 0.1 ms a tile: leaf-rich graph n = 130,001, 16 tiles of 64, 24.7 ms with the waits).
+  // A tile that failed (before any BC update) stops the ones behind it; it is run again, and the
+  // batch goes on from there, so BC takes the tiles in list order in any case.
+  int first = 0;  // sources done
+  static const bool tracing = getenv("BC_TRACE_FILE") != nullptr;
+  if (a.loop_mode == 0 && !a.out_depth && !tracing) {
+    bool ext = ws->ext_sticky;
+    int attempt = 0;
+    while (first < a.nsrc && !s) {
+      if (ext) {
+        s = ws_ext(ctx, ws);
+        if (!s) s = ws_hpart(ctx, ws, dg->nnz, hub, hub_chunk, true);
+        if (s) break;
+      }
+      TileSum *sums = (TileSum *)((char *)ws->stop + 16);
+      const KPtrs k = kptrs(G, ext);
+      cudaError_t e = cudaMemsetAsync(ws->stop, 0, 16, st);
+      if (e == cudaSuccess) e = cudaEventRecord(e0, st);
+      int cnt = 0;
+      for (int t0 = first; t0 < a.nsrc && cnt < kTileBatch && e == cudaSuccess && !s; t0 += a.T, cnt++) {
+        const int nt = std::min(a.nsrc - t0, a.T);
+        TK p = params(t0, nt);
+        p.stop = ws->stop;
+        k_wsrc<<<(a.T + 255) / 256, 256, 0, st>>>(p.src, nt, a.omega, ws->wsrc, a.T);
+        s = tile_clear(ws, G, st);
+        if (s) break;
+        int fo = 0;
+        void *args[] = {&p, &fo};
+        e = cudaLaunchCooperativeKernel(k.persistent, dim3(ctx->num_sms), dim3(k.tpb), args, 0, st);
+        if (e != cudaSuccess) break;
+        k_tile_end<<<1, 1, 0, st>>>(ws->ctl, ws->stop, sums + cnt);
+        e = cudaGetLastError();
+      }
+      if (e == cudaSuccess) e = cudaEventRecord(e1, st);
+      TileSum h[kTileBatch];
+      if (e == cudaSuccess && cnt > 0) e = cudaMemcpyAsync(h, sums, cnt * sizeof(TileSum), cudaMemcpyDeviceToHost, st);
+      const cudaError_t se = cudaStreamSynchronize(st);
+      if (e == cudaSuccess) e = se;
+      if (s) break;
+      if (e != cudaSuccess) {
+        s = cuda_fail(e, "tile batch");
+        break;
+      }
+      float ms = 0.f;
+      cudaEventElapsedTime(&ms, e0, e1);
+      total_ms += ms;
+      int derr = 0;
+      for (int i = 0; i < cnt; i++) {
+        if (h[i].err) {
+          derr = h[i].err;
+          break;
+        }
+        first = std::min(a.nsrc, first + a.T);
+        attempt = 0;
+        launches_total += 3;  // weights, tile, sums
+        levels_total += h[i].levels;
+        reached += (int64_t)h[i].reached;
+        reached_arcs += (int64_t)h[i].reached_arcs;
+        ovf_sources += h[i].ovf_sources;
+        maxd = std::max(maxd, h[i].lmax);
+      }
+      if (!derr) continue;
+      if (derr == BCD_NEEDEXT && !ext) {
+        ext = ws->ext_sticky = true;
+      } else if (derr == BCD_CAPACITY && ++attempt < 24) {
+        s = cudaMemsetAsync(ws->cand, 0, ((size_t)ws->n / 32 + 1) * 4, st) == cudaSuccess
+                ? ws_A(ctx, ws, ws->capA * 2) : fail(BC_ECUDA, "tile candidate bitmap");
+      } else if (derr == BCD_TIMEOUT) {
+        cudaMemsetAsync(ws->cand, 0, ((size_t)ws->n / 32 + 1) * 4, st);
+        cudaStreamSynchronize(st);
+        s = fail(BC_ETIMEDOUT, "tile kernel: a grid barrier wait passed its limit");
+      } else {
+        s = fail(BC_ECUDA, "tile kernel reported device error " + std::to_string(derr));
+      }
+    }
+  }
+  for (int t0 = first; t0 < a.nsrc && !s; t0 += a.T) {
     const int nt = a.nsrc - t0 < a.T ? a.nsrc - t0 : a.T;
     bool ext = ws->ext_sticky;
     for (int attempt = 0; attempt < 24; attempt++) {
@@ -2969,72 +3142,7 @@ bc_status tile_run(Ctx *ctx, Graph *g, TileWS **wsp, const TileArgs &a, cudaStre
         if (!s) s = ws_hpart(ctx, ws, dg->nnz, hub, hub_chunk, true);
         if (s) break;
       }
-      TK p;
-      memset(&p, 0, sizeof(p));
-      p.n = dg->n;
-      p.nnz = dg->nnz;
-      p.nsrc = nt;
-      p.rp = dg->rp;
-      p.ci = dg->ci;
-      p.omega = a.omega;
-      p.src = a.src + t0;
-      p.bc = a.bc;
-      p.leaf_term = a.omega != nullptr;
-      p.vis = ws->vis;
-      p.F = ws->F;
-      p.ovf = ws->ovf;
-      p.cand = ws->cand;
-      p.sig = ws->sig;
-      p.r = ws->r;
-      p.xm = ws->xm;
-      p.xe = ws->xe;
-      p.A = ws->A;
-      p.ACD = ws->ACD;
-      p.ARP = ws->ARP;
-      p.AM = ws->AM;
-      p.capA = ws->capA;
-      p.Aoff = ws->Aoff;
-      p.Lbits = ws->Lbits;
-      p.HE = ws->HE;
-      p.HEoff = ws->HEoff;
-      p.HEk = ws->HEk;
-      p.Hdone = ws->Hdone;
-      p.Hpart = ws->Hpart;
-      p.FPs = (unsigned long long *)ws->Hpart;
-      p.FPm = ws->FPm;
-      p.FPx = ws->FPx;
-      p.FPe = ws->FPe;
-      p.Fdone = ws->Fdone;
-      p.HPbu = ws->HPbu;
-      p.nhub_items = ws->nhub_items;
-      p.C = ws->C;
-      p.CPD = ws->CPD;
-      p.CRP = ws->CRP;
-      p.Ch = ws->Ch;
-      p.ChP = ws->ChP;
-      p.hubs = ws->hubs;
-      p.Lbu = ws->Lbu;
-      p.PDbu = ws->PDbu;
-      p.RPbu = ws->RPbu;
-      p.nhubs = ws->nhubs;
-      p.nbu = ws->nbu;
-      p.Ebu = ws->Ebu;
-      p.wsrc = ws->wsrc;
-      p.ctl = ws->ctl;
-      for (int gi = 0; gi < 8; gi++) {
-        uint32_t m = 0;
-        for (int b = 0; b < 32; b++)
-          if (gi * 32 + b >= nt) m |= 1u << b;
-        p.unused[gi] = m;
-      }
-      p.alpha = a.alpha;
-      p.beta = a.beta;
-      p.hub = hub;
-      p.hub_chunk = hub_chunk;
-      p.nreq = a.nreq;
-      p.lane_req = a.lane_req ? a.lane_req + t0 : nullptr;
-      p.req_bc = a.req_bc;
-      p.limit_ns = ctx->wait_limit_ns;
+      TK p = params(t0, nt);
       static const char *trace_file = getenv("BC_TRACE_FILE");
       if (trace_file && !trace_buf) {
         if (cudaMalloc(&trace_buf, (size_t)(1 << 20) * 16) != cudaSuccess) {
