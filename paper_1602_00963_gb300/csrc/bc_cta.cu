@@ -1101,8 +1101,9 @@ struct CtaPlan {
 //   scale 12 all sources 3.3 against 4.1 with 128 registers and 512 threads; social graph above
 //   10.0 against 10.7), else 128 registers and 512 threads (G(9000, 36,000) all sources 9.0
 //   against 10.0), a lane then taking rows of up to 32 arcs instead of 12 (G(9000, 72,000): 12.9,
-//   with 16 16.4, with 12 20.5; the social graph 9.6 with 12, 9.9 with 16, 11.1 with 32).  From global memory 128 registers (64 spill in the sweeps: grid 1024^2
-//   92 against 70); narrow graphs need no code for larger rows and run with 80 (59).
+//   with 16 16.4, with 12 20.5; the social graph 9.6 with 12, 9.9 with 16, 11.1 with 32).  From
+//   global memory 128 registers (64 spill in the sweeps: grid 1024^2 92 against 70); narrow
+//   graphs need no code for larger rows and run with 80 (59).
 // * Threads: an SM's threads over the states that fit it and have a source (one source on
 //   n = 1000: 85 us with 512, 95 with 128); from global memory 512 (social graph
 //   n = 60,001, 500 sources: 11.9, 13.3 with 256), narrow graphs 96 / 192 / 384 by size (grid
