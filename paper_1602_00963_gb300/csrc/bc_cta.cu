@@ -337,15 +337,30 @@ __device__ __forceinline__ void fwd_append(const CtaState<SM> &S, const FwdLevel
   }
 }
 
-// Claim x for the next level; true for the one thread that does.
-__device__ __forceinline__ bool fwd_claim(const CtaState<true> &S, const FwdLevel &f, int x) {
-  const uint32_t bit = 1u << (x & 31);
-  if (atomicOr(&S.vis[x >> 5], bit) & bit) return false;
-  *(volatile uint16_t *)&S.tag[x] = (uint16_t)(f.tl + 2u);
-  return true;
+// Claim the K vertices flagged in un for the next level: nw[k] for the one thread that does.  The
+// claims are all on their way before the first answer is looked at (an answer from L2 takes as
+// long as the records' loads).
+template <int K>
+__device__ __forceinline__ void fwd_claim(const CtaState<true> &S, const FwdLevel &f, const bool (&un)[K],
+                                          const int (&x)[K], bool (&nw)[K]) {
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    const uint32_t bit = 1u << (x[k] & 31);
+    nw[k] = un[k] && !(atomicOr(&S.vis[x[k] >> 5], bit) & bit);
+    if (nw[k]) *(volatile uint16_t *)&S.tag[x[k]] = (uint16_t)(f.tl + 2u);
+  }
 }
-__device__ __forceinline__ bool fwd_claim(const CtaState<false> &S, const FwdLevel &f, int x) {
-  return atomicMax(&S.rec[x].tag, f.tl + 2u) < f.t0;
+template <int K>
+__device__ __forceinline__ void fwd_claim(const CtaState<false> &S, const FwdLevel &f, const bool (&un)[K],
+                                          const int (&x)[K], bool (&nw)[K]) {
+  uint32_t old[K];
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    old[k] = ~0u;
+    if (un[k]) old[k] = atomicMax(&S.rec[x[k]].tag, f.tl + 2u);
+  }
+#pragma unroll
+  for (int k = 0; k < K; k++) nw[k] = old[k] < f.t0;
 }
 
 // Store w's sigma: s modulo 2^64, or (ov: it passed 2^64) its extended range a.
@@ -395,7 +410,7 @@ __device__ __forceinline__ void fwd_groups(const CtaK &p, const CtaState<SM> &S,
     bool ov = false;
     for (int u = 0; u < steps; u += W * UN) {
       int x[UN];
-      bool nw[UN];
+      bool nw[UN], un[UN];
 #pragma unroll
       for (int k = 0; k < UN; k++) x[k] = u + k * W + sub < dg ? p.ci[ee + u + k * W + sub] : -1;
       Rec r[UN];
@@ -405,10 +420,11 @@ __device__ __forceinline__ void fwd_groups(const CtaK &p, const CtaState<SM> &S,
         if (x[k] >= 0) r[k] = cta_rec(S, x[k], tp, false);
       }
 #pragma unroll
-      for (int k = 0; k < UN; k++) {
-        nw[k] = unreached<SM>(f, r[k].tag) && fwd_claim(S, f, x[k]);
+      for (int k = 0; k < UN; k++) un[k] = unreached<SM>(f, r[k].tag);
+      fwd_claim(S, f, un, x, nw);
+#pragma unroll
+      for (int k = 0; k < UN; k++)
         if ((r[k].tag & ~1u) == tp) sum_carry(s, ov, r[k].val, r[k].tag & 1u);
-      }
       fwd_append<SM, UN>(S, f, nw, x);
     }
 #pragma unroll
@@ -534,28 +550,42 @@ __device__ __forceinline__ int cta_forward(const CtaK &p, const CtaState<SM> &S,
         int x[4];
         row_arcs<SM>(p, row, u, dl, x);
         Rec r[4];
-        bool nw[4];
+        bool nw[4], un[4];
 #pragma unroll
         for (int j = 0; j < 4; j++) {
           r[j].tag = f.tl;  // neither a parent nor a successor
           if (u < dl && x[j] >= 0) r[j] = cta_rec(S, x[j], tp, ext);
         }
 #pragma unroll
+        for (int j = 0; j < 4; j++) un[j] = unreached<SM>(f, r[j].tag);
+        fwd_claim(S, f, un, x, nw);
+        // the parents' sums while the claims are on their way
+        bool allx = true;  // every parent is in the extended range
+#pragma unroll
         for (int j = 0; j < 4; j++) {
-          const bool un = unreached<SM>(f, r[j].tag);
-          nw[j] = un && fwd_claim(S, f, x[j]);
-          if (!SM && (un || r[j].tag == tn) && u < 8) succ |= 1 << (u + j);
+          if (!SM && (un[j] || r[j].tag == tn) && u < 8) succ |= 1 << (u + j);
+          if ((r[j].tag & ~1u) == tp) {
+            sum_carry(sum, ov, r[j].val, r[j].tag & 1u);
+            allx = allx && (r[j].tag & 1u);
+          }
         }
-        fwd_append<SM, 4>(S, f, nw, x);
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-          if ((r[j].tag & ~1u) == tp) sum_carry(sum, ov, r[j].val, r[j].tag & 1u);
         if (!SM && ov && !xp && row.deg <= kThin) {
+          if (allx) {  // mantissas brought to the largest exponent (exact) and added in arc order
+            a.e = INT_MIN;
 #pragma unroll
-          for (int j = 0; j < 4; j++)
-            if ((r[j].tag & ~1u) == tp) xs_add(a, rec_sigma(r[j]));
+            for (int j = 0; j < 4; j++)
+              if ((r[j].tag & ~1u) == tp) a.e = max(a.e, r[j].e);
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+              if ((r[j].tag & ~1u) == tp) a.m += scale2(__longlong_as_double((long long)r[j].val), r[j].e - a.e);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+              if ((r[j].tag & ~1u) == tp) xs_add(a, rec_sigma(r[j]));
+          }
           a = xs_norm(a);
         }
+        fwd_append<SM, 4>(S, f, nw, x);
       }
       if constexpr (LD > kNarrowDeg) {
         constexpr int GD = LD > kGroupDeg ? LD : kGroupDeg;
@@ -1090,7 +1120,8 @@ struct CtaPlan {
   const void *kernel = nullptr;
 };
 
-// The rule, and both sides of its lines (ms per call, this GPU):
+// The rule, and both sides of its lines (ms per call, this GPU, a pair on the same code; the grids
+// went from 5.5 and 59 to 4.9 and 53 when a level's claims were sent together):
 // * State in shared memory where it fits (n <= 22,654): G(n, 4n) n = 16,384, 500 sources 1.15
 //   against 1.79 from global memory, social graph n = 20,001, 3000 sources 9.9 against 16.3.
 //   Narrow graphs (largest degree <= 8, road-like: levels of about sqrt(n) vertices) only while
