@@ -62,8 +62,8 @@ enum {
 /* (by default the per-source path runs graphs of up to 65,536 vertices one source per CTA,
  *  all SMs on different sources; larger graphs use the grid-wide kernel, one source at a
  *  time over the whole GPU, unless BC_PLAIN_CTA or the autotuner picks the per-CTA kernel,
- *  which suits sparse high-diameter graphs; it holds 48 bytes per vertex per CTA, two CTAs
- *  per SM, for graphs of up to 2^24 vertices) */
+ *  which suits sparse high-diameter graphs; it holds 32 bytes per vertex per CTA, one to eight
+ *  CTAs per SM by size, and 16 bytes per vertex once, for graphs of up to 2^24 vertices) */
 /* bc_exact: 2-degree heuristic (Sec. 3.4.2).  A set of degree-2 vertices c, no two sharing
  * a neighbour or being one, is run without a traversal of its own: the shortest-path DAG of c
  * is derived from those of its two neighbours a, b (run from the same CTA) and c's

@@ -960,7 +960,7 @@ bc_status plain_setup(int *blocks_per_sm) {
 
 int64_t plain_bytes(int32_t n) {
   int64_t N = n + 2, nw = (n + 31) / 32 + 1;
-  return N * (4 * 5 + 8 * 6) + nw * 4 * 3 + (int64_t)sizeof(PlainCtl) + 4096;
+  return N * (4 * 5 + 8 * 6) + nw * 4 * 3 + (int64_t)sizeof(PlainCtl) + 4032;
 }
 
 void plain_free(Ctx *ctx, PlainWS *ws) {
