@@ -779,28 +779,6 @@ __device__ __forceinline__ void fwd_hits_add(const TK &p, const FwdHit<G, EXT> &
   }
   // 64-bit mode (EXT is handled above): an overflowed parent has already flagged the tile
   // for the extended rerun, so only the additions' carries are checked
-  if constexpr (G == 4) {  // straight-line: no branch but the row load's (see bwd_hits_add)
-    const uint32_t me = 1u << lane;
-    while (hd) {
-      const int jj = __ffs(hd) - 1;
-      hd &= hd - 1;
-      const int pn = __shfl_sync(BC_FULL, h.pj, jj);
-      uint32_t m[G], u = 0u;
-#pragma unroll
-      for (int g = 0; g < G; g++) {
-        m[g] = __shfl_sync(BC_FULL, h.bm[g], jj);
-        u |= m[g];
-        a.newm[g] |= m[g];
-      }
-      unsigned long long sv[G];
-#pragma unroll
-      for (int g = 0; g < G; g++) sv[g] = 0ull;
-      if (u & me) load_lane<G>(p.sig + sidx<G>(pn, 0, lane), sv);
-#pragma unroll
-      for (int g = 0; g < G; g++) add_carry(a.s[g], a.cy, (m[g] & me) ? sv[g] : 0ull);
-    }
-    return;
-  }
   while (hd) {
     unsigned long long sv[HB<G>::value][G];
     uint32_t mq[HB<G>::value][G];
@@ -1807,36 +1785,6 @@ __device__ __forceinline__ void bwd_hits_add(const TK &p, const BwdHit<G, EXT> &
     FF2 acc2[G / 2];
 #pragma unroll
     for (int j = 0; j < G / 2; j++) acc2[j] = ff2_pack(o.acc[2 * j], o.acc[2 * j + 1]);
-    // Tiles of 128 are bound by issue: 22 M dense hits a sweep and tile at 35 of 128 sources on
-    // average.  One row at a time, masks as single-bit tests, both pairs added always: a branch
-    // around a pair without sources costs more than the additions it saves (with this and the
-    // forward loop like it 10.09 ms per tile of 128 against 10.24; tiles of 256, which spill more,
-    // 24.7 against 23.7, keep the loop below; rows through shared memory by cp.async 11.9, whose
-    // extra instructions outweighed the latency they hid).
-    if constexpr (G == 4) {
-      const uint32_t me = 1u << lane;
-      while (hd) {
-        const int jj = __ffs(hd) - 1;
-        hd &= hd - 1;
-        const int vq = __shfl_sync(BC_FULL, h.v, jj);
-        uint32_t m[G], u = 0u;
-#pragma unroll
-        for (int g = 0; g < G; g++) {
-          m[g] = __shfl_sync(BC_FULL, h.bm[g], jj);
-          u |= m[g];
-        }
-        float2 x[G];
-#pragma unroll
-        for (int g = 0; g < G; g++) x[g] = make_float2(0.0f, 0.0f);
-        if (u & me) load_lane<G>(p.r + sidx<G>(vq, 0, lane), x);
-#pragma unroll
-        for (int j = 0; j < G / 2; j++) {
-          if (!(m[2 * j] & me)) x[2 * j] = make_float2(0.0f, 0.0f);
-          if (!(m[2 * j + 1] & me)) x[2 * j + 1] = make_float2(0.0f, 0.0f);
-          ff2_add(acc2[j], ff2_pack(x[2 * j], x[2 * j + 1]));
-        }
-      }
-    }
     while (hd) {
       FF2 xq[HB<G>::value][G / 2];
       uint32_t mq[HB<G>::value][G];
