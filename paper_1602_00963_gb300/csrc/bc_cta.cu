@@ -678,7 +678,7 @@ template <bool SM, int LD, bool EXT>
 __device__ __forceinline__ void cta_backward(const CtaK &p, const CtaState<SM> &S, int s, int lmax, double *bcp,
                                              CtaShared &sh) {
   const int tid = threadIdx.x, slot = cta_slot(p);
-  const float2 wsrc = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[s] : 0ull));
+  const float2 wsrc = ff_u64_bits(1ull + (p.omega ? (unsigned long long)p.omega[s] : 0ull));
   int hi = S.loff[lmax + 1], lo = S.loff[lmax];
   int qe = -1;
   Row row = no_row();
@@ -717,10 +717,10 @@ __device__ __forceinline__ void cta_backward(const CtaK &p, const CtaState<SM> &
       int ew = 0;
       if (EXT) {
         const XS x = rec_sigma(own);
-        mw = ff_mant(x.m);
+        mw = ff_mant_bits(x.m);
         ew = x.e;
       } else {
-        mw = ff_u64(own.val);
+        mw = ff_u64_bits(own.val);
       }
       if (dd < lmax) {
         const int dl = row.deg <= LD ? row.deg : 0;
@@ -748,7 +748,7 @@ __device__ __forceinline__ void cta_backward(const CtaK &p, const CtaState<SM> &
         }
       }
       if (qe != -1) {
-        const float2 om1 = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull));
+        const float2 om1 = ff_u64_bits(1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull));
         float2 rw = ff_mul(om1, ff_rcp(mw));
         ff_add(rw, acc);
         if constexpr (SM) {
@@ -815,7 +815,7 @@ __device__ __forceinline__ void cta_backward_deg2(const CtaK &p, const CtaState<
                                                   CtaShared &sh) {
   const int lane = lane_id(), slot = cta_slot(p);
   const int lmax = 1 + (lmaxA > lmaxB ? lmaxA : lmaxB);
-  const float2 wsrc = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[c] : 0ull));
+  const float2 wsrc = ff_u64_bits(1ull + (p.omega ? (unsigned long long)p.omega[c] : 0ull));
   for (int D = lmax; D >= 1; --D) {
     const uint32_t tc = (C.base + (uint32_t)D) << 1, tn = tc + 2u;
 #pragma unroll 1
@@ -842,11 +842,11 @@ __device__ __forceinline__ void cta_backward_deg2(const CtaK &p, const CtaState<
               xs_add(x, rec_sigma(rb));
               x = xs_norm(x);
             }
-            mw = ff_mant(x.m);
+            mw = ff_mant_bits(x.m);
             ew = x.e;
           } else {
-            mw = ff_u64(side ? rb.val : ra.val);
-            if (da == db) ff_add(mw, ff_u64(rb.val));
+            mw = ff_u64_bits(side ? rb.val : ra.val);
+            if (da == db) ff_add(mw, ff_u64_bits(rb.val));
           }
         }
         float2 acc = make_float2(0.0f, 0.0f);
@@ -884,7 +884,7 @@ __device__ __forceinline__ void cta_backward_deg2(const CtaK &p, const CtaState<
           }
         }
         if (mine) {
-          const float2 om1 = ff_u64(1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull));
+          const float2 om1 = ff_u64_bits(1ull + (p.omega ? (unsigned long long)p.omega[w] : 0ull));
           float2 rw = ff_mul(om1, ff_rcp(mw));
           ff_add(rw, acc);
           Rec r;
