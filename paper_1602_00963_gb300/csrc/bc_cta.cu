@@ -569,7 +569,9 @@ __device__ __forceinline__ int cta_forward(const CtaK &p, const CtaState<SM> &S,
             allx = allx && (r[j].tag & 1u);
           }
         }
-        if (!SM && ov && !xp && row.deg <= kThin) {
+        // u < dl: this row's own step.  The loop goes on for longer rows of the warp, and a step
+        // without parents would leave the sum with the exponent of none.
+        if (!SM && u < dl && ov && !xp && row.deg <= kThin) {
           if (allx) {  // mantissas brought to the largest exponent (exact) and added in arc order
             a.e = INT_MIN;
 #pragma unroll
