@@ -19,8 +19,8 @@
 // range needs no pass of its own); neighbours not reached yet are claimed for level l + 1 by
 // an atomic maximum on their level and queued.  The levels carry the source's base, which
 // grows by the levels used, so records of earlier sources read as "not reached" and nothing is
-// reset between sources.  An entry of degree <= 4 notes which neighbours are its successors in
-// its queue entry, so the backward sweep loads those alone.
+// reset between sources.  With state in global memory a queue entry notes which of the first eight
+// arcs of a row handled by a lane lead to successors, so the backward sweep leaves the others' records alone.
 // Backward level d: a vertex sums its successors' r in float-float arithmetic, delta = sigma *
 // sum, r = (1 + omega) / sigma + sum, and the CTA's BC partial grows by (omega[s] + 1) * delta.
 // When a sigma of the source passed 2^64 sigma is taken as m 2^e (m in [0.5, 1)) and r is kept
@@ -46,7 +46,13 @@ constexpr int kGroupDeg = 32;   // above a lane's degree: eight lanes up to here
 constexpr int kNarrowDeg = 8;   // graphs of at most this degree: lanes alone (no code for larger rows)
 constexpr uint32_t kBase0 = 2;  // first base: level base - 1 is never in use, nor 0
 constexpr uint32_t kBaseMax = 0x3f000000u;
-constexpr int kIdMask = 0xffffff;  // queue entries: vertex id (n <= 2^24), successor bits above
+// Queue entries: vertex id (n <= 2^24), above it a bit for each of the row's first eight arcs that leads
+// to a successor.  No entry may equal -1, the mark of a missing one, whatever its id: in narrow
+// graphs one of a row's arcs, at most eight, leads to a parent; else the eighth arc's bit stays clear
+// and its record is always read.
+constexpr int kIdMask = 0xffffff;
+template <int LD>
+constexpr bool kSeven = LD > kNarrowDeg;
 constexpr size_t kCtaSmemMax = 224 * 1024;  // state kept in shared memory up to this
 
 struct CtaK {
@@ -602,7 +608,7 @@ __device__ __forceinline__ int cta_forward(const CtaK &p, const CtaState<SM> &S,
         if (xs) a = y;
       }
       if (in) {
-        if (!SM) S.Q[i] = w | succ << 24;
+        if (!SM) S.Q[i] = w | (kSeven<LD> ? succ & 0x7f : succ) << 24;
         if (l > 0) fwd_commit(S, f, w, sum, ov, xp, a);  // the source keeps sigma = 1
         if (ov) sh.ovf = 1;
       }
@@ -726,7 +732,7 @@ __device__ __forceinline__ void cta_backward(const CtaK &p, const CtaState<SM> &
       }
       if (dd < lmax) {
         const int dl = row.deg <= LD ? row.deg : 0;
-        const unsigned succ = SM ? 0u : (unsigned)qe >> 24;
+        const unsigned succ = SM ? 0u : (unsigned)qe >> 24 | (kSeven<LD> ? 0x80u : 0u);
         for (int u = 0; u < dl; u += 4) {
           int x[4];
           row_arcs<SM>(p, row, u, dl, x);
