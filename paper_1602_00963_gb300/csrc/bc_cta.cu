@@ -853,8 +853,7 @@ __device__ __forceinline__ void cta_backward_deg2(const CtaK &p, const CtaState<
             mw = ff_mant_bits(x.m);
             ew = x.e;
           } else {
-            mw = ff_u64_bits(side ? rb.val : ra.val);
-            if (da == db) ff_add(mw, ff_u64_bits(rb.val));
+            mw = ff_sum_u64(side ? rb.val : ra.val, da == db ? rb.val : 0ull);
           }
         }
         float2 acc = make_float2(0.0f, 0.0f);

@@ -127,6 +127,14 @@ __device__ __forceinline__ float2 ff_u64_bits(unsigned long long s) {
   const float lo = __uint2float_rn((unsigned)(t >> 16) & 0xffffffu) * pow2f(e - 47);
   return ff_norm(hi, lo);
 }
+// a + b (not both 0; the sum may pass 2^64), added as integers and truncated once, as ff_u64 truncates
+__device__ __forceinline__ float2 ff_sum_u64(unsigned long long a, unsigned long long b) {
+  const unsigned long long s = a + b;
+  const bool c = s < a;
+  const float2 x = ff_u64_bits(c ? s >> 1 | 1ull << 63 : s);
+  const float k = c ? 2.0f : 1.0f;
+  return make_float2(x.x * k, x.y * k);
+}
 // an extended-range mantissa m in [0.5, 1): its 53 bits' top 24 and the next 24, as ff_u64 takes them
 __device__ __forceinline__ float2 ff_mant_bits(double m) {
   const unsigned long long f = (unsigned long long)__double_as_longlong(m) & (unsigned long long)kFFMantBits;
