@@ -1097,10 +1097,10 @@ __global__ void k_cta_reduce_req(const double *bcp, int nreq, const int32_t *rc,
 }  // namespace
 
 struct CtaWS {
-  int n = 0, ncta = 0;
-  int kind = -1;       // slice layout of the last completed launch: 0 global, 1 shared, 2 triples
-  bool clean = false;  // the slices' bases and records are valid for that layout
-  size_t slice = 0;    // bytes per CTA
+  int n = 0, rows = 0;  // BC partials (CTAs) that bcp holds
+  int kind = -1;        // slice layout of the last completed launch: 0 global, 1 shared, 2 triples
+  int clean = 0;        // slices (CTAs from 0 on) whose bases and records are valid for that layout
+  size_t b_gws = 0;     // bytes of gws, cut into slices of the layout of each launch
   double *bcp = nullptr;
   char *gws = nullptr;
   int4 *row4 = nullptr;  // row records (null: they did not fit the HBM budget)
@@ -1195,34 +1195,13 @@ static bc_status cta_plan(Ctx *ctx, int n, int max_degree, int units, bool tri, 
   return BC_OK;
 }
 
-// A workspace of min(plan's CTAs, CTAs the call can use) slices for graphs of n vertices.
-static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, int64_t units, const CtaPlan &pl) {
-  CtaWS *ws = *wsp;
-  // sizes of the largest layout (with triples only once a call has them)
-  const bool tri = pl.kind == 2;
-  size_t slice = 16 + cta_state_bytes(n, false) * (tri ? 2 : 1) + (tri ? (size_t)n * 16 : 0);
-  if (pl.kind == 1) slice = 16 + cta_state_bytes(n, true);
-  slice = (slice + 255) & ~(size_t)255;
-  const size_t per_cta = (size_t)n * 8 + slice;
-  int ncta = (int)std::min<int64_t>(pl.ncta, std::max<int64_t>(units, 32));
-  if (ctx->mem.budget) {  // fewer CTAs when the context's HBM budget is tight: at most half
-    // of what is free, so that requests arriving meanwhile still find room (serving)
-    const size_t used = ctx->mem.used.load() - (ws ? ws->bytes : 0);
-    const size_t avail = ctx->mem.budget > used + 64 ? ctx->mem.budget - used - 64 : 0;
-    ncta = (int)std::min<size_t>((size_t)ncta, std::max<size_t>(avail / 2 / per_cta, avail >= per_cta ? 1 : 0));
-    if (ncta < 1) return fail(BC_ENOMEM, "CTA per-source workspace exceeds the context HBM budget");
-  }
-  if (ws && ws->n == n && ws->ncta >= ncta && ws->slice >= slice) return BC_OK;
-  if (ws) {
-    cta_free(ctx, ws);
-    *wsp = nullptr;
-  }
-  ws = new (std::nothrow) CtaWS();
+static bc_status cta_alloc(Ctx *ctx, CtaWS **wsp, int n, int rows, size_t b_gws, bool row4) {
+  CtaWS *ws = new (std::nothrow) CtaWS();
   if (!ws) return fail(BC_ENOMEM, "host allocation failed");
   ws->n = n;
-  ws->ncta = ncta;
-  ws->slice = slice;
-  const size_t b_bcp = (size_t)ncta * n * 8, b_gws = slice * ncta, b_row = pl.kind == 1 ? 0 : (size_t)n * 16;
+  ws->rows = rows;
+  ws->b_gws = b_gws;
+  const size_t b_bcp = (size_t)rows * n * 8, b_row = row4 ? (size_t)n * 16 : 0;
   ws->bytes = b_bcp + b_gws + 64 + 2 * (kCtaMaxReq + 1) * sizeof(int32_t);
   bc_status s = ctx->mem.alloc(nullptr, ws->bytes);
   if (s) {
@@ -1253,6 +1232,56 @@ static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, int64_t units, const C
   return BC_OK;
 }
 
+// Bytes of a CTA's slice in a plan's layout (a second state and c's records only with triples).
+static size_t cta_slice(const CtaPlan &pl, int n) {
+  size_t slice = 16 + cta_state_bytes(n, pl.kind == 1);
+  if (pl.kind == 2) slice += cta_state_bytes(n, false) + (size_t)n * 16;
+  return (slice + 255) & ~(size_t)255;
+}
+
+// A workspace for min(plan's CTAs, CTAs the call can use) in the plan's layout, *max_cta = how many it
+// holds.  It grows to at least twice the CTAs (calls whose number of sources grows one by one would
+// free and allocate it each time: k = 33 to 150 on n = 60,000 took 118 allocations, now at most 4) and keeps
+// what other layouts needed (one- and two-state calls taking turns), as far as half of the
+// context's free budget, else the device's memory, allows.
+static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, int64_t units, const CtaPlan &pl, int *max_cta) {
+  CtaWS *ws = *wsp;
+  const size_t slice = cta_slice(pl, n), per_cta = (size_t)n * 8 + slice;
+  const bool same = ws && ws->n == n;
+  const int have = same ? (int)std::min<size_t>({(size_t)ws->rows, ws->b_gws / slice, (size_t)pl.ncta}) : 0;
+  int ncta = (int)std::min<int64_t>(pl.ncta, std::max<int64_t>(units, 32));
+  size_t room = SIZE_MAX;
+  if (ctx->mem.budget) {  // fewer CTAs when the context's HBM budget is tight: at most half
+    // of what is free, so that requests arriving meanwhile still find room (serving)
+    const size_t used = ctx->mem.used.load() - (ws ? ws->bytes : 0);
+    const size_t avail = ctx->mem.budget > used + 64 ? ctx->mem.budget - used - 64 : 0;
+    room = avail / 2;
+    ncta = (int)std::min<size_t>((size_t)ncta, std::max<size_t>(room / per_cta, avail >= per_cta ? 1 : 0));
+    if (ncta < 1) return fail(BC_ENOMEM, "CTA per-source workspace exceeds the context HBM budget");
+  }
+  *max_cta = have;
+  if (have >= ncta) return BC_OK;
+  int rows = ncta;
+  size_t b_gws = slice * ncta;
+  bool row4 = pl.kind != 1;
+  if (same) {
+    const int grown = std::max(ncta, (int)std::min<size_t>({(size_t)pl.ncta, (size_t)2 * have, room / per_cta}));
+    const int r2 = std::max(grown, ws->rows);
+    const size_t g2 = std::max(slice * grown, ws->b_gws);
+    if ((size_t)r2 * n * 8 + g2 <= room) {
+      rows = r2;
+      b_gws = g2;
+    }
+    row4 = row4 || ws->row4;
+  }
+  cta_free(ctx, ws);
+  *wsp = nullptr;
+  bc_status s = cta_alloc(ctx, wsp, n, rows, b_gws, row4);
+  if (s && (rows != ncta || b_gws != slice * ncta)) s = cta_alloc(ctx, wsp, n, ncta, slice * ncta, row4);
+  if (!s) *max_cta = (int)std::min<size_t>({(size_t)(*wsp)->rows, (*wsp)->b_gws / slice, (size_t)pl.ncta});
+  return s;
+}
+
 bool cta_fits(int32_t n) { return n > 0 && n <= kCtaMaxN; }
 
 bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStream_t st, bc_stats *acc) {
@@ -1263,10 +1292,10 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   CtaPlan pl;
   const int units = sssp ? 1 : std::max(a.nsrc, a.ntri);
   bc_status s = cta_plan(ctx, n, a.max_degree, units, !sssp && a.ntri > 0, &pl);
-  if (!s) s = cta_ensure(ctx, wsp, n, units, pl);
+  int max_cta = 0;
+  if (!s) s = cta_ensure(ctx, wsp, n, units, pl, &max_cta);
   if (s) return s;
   CtaWS *ws = *wsp;
-  const int max_cta = std::min(pl.ncta, ws->ncta);
   CtaK p;
   memset(&p, 0, sizeof(p));
   p.n = n;
@@ -1278,7 +1307,7 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   p.leaf_term = a.leaf_term ? 1 : 0;
   p.bcp = ws->bcp;
   p.gws = ws->gws;
-  p.slice = ws->slice;
+  p.slice = cta_slice(pl, n);
   p.row4 = pl.kind == 1 ? nullptr : ws->row4;
   p.spread = a.max_degree <= 0 || a.max_degree > kThin;
   p.stats = ws->stats;
@@ -1298,13 +1327,13 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   BC_CUDA_TRY(cudaEventCreate(&e0));
   BC_CUDA_TRY(cudaEventCreate(&e1));
   cudaEventRecord(e0, st);
-  const bool was_clean = ws->clean && ws->kind == pl.kind;
-  ws->clean = false;  // until the launches are known to have completed
+  const int was_clean = ws->kind == pl.kind ? ws->clean : 0;
+  ws->clean = 0;  // until the launches are known to have completed
   if (p.row4) k_cta_rows<<<ctx->num_sms * 4, 256, 0, st>>>(n, dg->rp, dg->ci, ws->row4);
   cudaError_t le = cudaSuccess;
   auto launch = [&](const CtaK &kp, int ncta, const int32_t *rc, double *const *rbc) {
     CtaK q = kp;
-    q.clean = (was_clean || launched_max >= ncta) ? 1 : 0;
+    q.clean = std::max(was_clean, launched_max) >= ncta ? 1 : 0;
     void *args[] = {&q};
     le = cudaLaunchKernel(pl.kernel, dim3(ncta), dim3(pl.threads), args, pl.smem, st);
     launched_max = std::max(launched_max, ncta);
@@ -1394,7 +1423,7 @@ bc_status cta_run(Ctx *ctx, Graph *g, CtaWS **wsp, const PlainArgs &a, cudaStrea
   if (se != cudaSuccess) return cuda_fail(se, "CTA per-source kernel");
   BC_CUDA_TRY(cudaStreamSynchronize(st));
   // the launched CTAs left their state cleared; CTAs not launched kept theirs
-  ws->clean = was_clean || launched_max == ws->ncta;
+  ws->clean = std::max(was_clean, launched_max);
   ws->kind = pl.kind;
   if (acc) {
     acc->seconds += ms * 1e-3;
