@@ -76,8 +76,8 @@ enum {
 /* bc_exact / bc_sources, grid-wide per-source kernel only (needs BC_PATH_PLAIN |
  * BC_PLAIN_GRID, else BC_EINVAL): the backward sweep scans each level's degree prefix CD
  * again instead of reusing the one the forward sweep stored (Sec. 3.1's reuse switched off,
- * for measuring it).  The prefix values are the same, so the result differs only by the
- * order of the kernel's floating-point atomic additions. */
+ * for measuring it); which levels it sums over their own arcs and which over the next level's
+ * stays as without the flag.  The prefix values and the result are the same bit for bit. */
 #define BC_NO_CD_REUSE    (1u << 14)
 /* bc_exact / bc_sources: the result depends only on the graph, the sources, the flags and
  * the GPU model (reading R9 of Eq. 2's sums: a fixed summation order, so repeated runs agree

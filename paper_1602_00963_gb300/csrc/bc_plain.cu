@@ -619,13 +619,12 @@ __device__ __forceinline__ int cta_excl_scan(int x, int *total, int *s_warp) {
   return r;
 }
 
-// Sec. 3.1 without its reuse (the ablation BC_NO_CD_REUSE): before the backward sweep reads
+// Sec. 3.1 without its reuse (the ablation BC_NO_CD_REUSE): before the backward sweep first reads
 // the degree prefix CD of level d's entries Q[q0, q1), it is scanned again instead of taken
 // from the forward appends.  CTAs sum the degrees of equal chunks of the level, then each
 // scans its chunk starting from E0 plus the sums of the CTAs before it.  The values equal
 // the stored ones (the appends lay entries and their edge offsets out in queue order), so
-// only the time differs (and the order of the backward's atomic additions).  Two grid
-// barriers.
+// only the time differs.  Two grid barriers.
 __device__ bool rescan_level(const PK &p, GridSync *gs, int d, int q0, int q1, int E0) {
   __shared__ int s_warp[kWarps + 1];
   __shared__ int s_base;
@@ -838,11 +837,17 @@ __device__ __forceinline__ void plain_body(const PK &p, unsigned char *smem) {
         else
           finalize_level<false>(p, a0, a1, ws, gtid, nthr);
         if (!phase_sync<SOLO>(p, gs, 4, D)) return;
+        bool pulled = false;
         for (int d = D - 1; d >= 1; --d) {
           const int b0 = p.lvl_off[d], b1 = a0, g0 = p.lvl_eoff[d], g1 = f0;
-          if (!SOLO && p.no_cd_reuse && !rescan_level(p, gs, d, b0, b1, g0)) return;
           // a pushed arc that leads back costs its own atomics, so push only from far fewer arcs
-          const bool push = !p.no_cd_reuse && (long long)(f1 - f0) * kPushFactor <= (long long)(g1 - g0);
+          const bool push = (long long)(f1 - f0) * kPushFactor <= (long long)(g1 - g0);
+          // the prefix that this step reads: the next level's when it pushes, unless the step before
+          // pulled and so had it scanned
+          if (!SOLO && p.no_cd_reuse && !(push && pulled) &&
+              !rescan_level(p, gs, push ? d + 1 : d, push ? a0 : b0, push ? a1 : b1, push ? f0 : g0))
+            return;
+          pulled = !push;
           if (push) {
             if (ext)
               push_level<true>(p, W, base + d, a0, a1, f0, f1, gwarp, nwarps);
