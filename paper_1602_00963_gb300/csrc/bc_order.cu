@@ -77,17 +77,21 @@ bc_status build_cache(Graph *g, const DeviceGraph *dg, int T, cudaStream_t st, T
   const int32_t n = dg->n;
   oc->rp = dg->rp;
   oc->L = 0;
+  if (dg->nnz == 0) return BC_OK;
   // the landmarks: a seeded sample of the non-isolated vertices in increasing order, picked on the
   // device by rank (flags, exclusive scan, one search per landmark)
   const size_t n1 = (size_t)n + 1, b_arr = (n1 * 4 + 255) & ~(size_t)255;
+  const size_t b_tmp = 2 * b_arr + 256 + scan_scratch_bytes((int64_t)n1);
   char *tmp = nullptr;
-  cudaError_t ce = cudaMalloc(&tmp, 2 * b_arr + 256 + scan_scratch_bytes((int64_t)n1));
+  bc_status s = c->mem.alloc((void **)&tmp, b_tmp);
+  if (s) {
+    oc->rp = nullptr;
+    return s;
+  }
   int32_t *flag = (int32_t *)tmp, *pos = (int32_t *)(tmp + b_arr), *pick = (int32_t *)(tmp + 2 * b_arr);
   int32_t pool = 0;
-  if (ce == cudaSuccess) {
-    k_lm_flags<<<c->num_sms * 4, 256, 0, st>>>(n, dg->rp, flag);
-    ce = scan_exclusive_i32(flag, pos, (int64_t)n1, tmp + 2 * b_arr + 256, st);
-  }
+  k_lm_flags<<<c->num_sms * 4, 256, 0, st>>>(n, dg->rp, flag);
+  cudaError_t ce = scan_exclusive_i32(flag, pos, (int64_t)n1, tmp + 2 * b_arr + 256, st);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(&pool, pos + n, 4, cudaMemcpyDeviceToHost, st);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
   const int L = (int)std::min<int64_t>(kLandmarks, pool);
@@ -100,7 +104,7 @@ bc_status build_cache(Graph *g, const DeviceGraph *dg, int T, cudaStream_t st, T
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(lm.data(), pick, (size_t)L * 4, cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
   }
-  if (tmp) cudaFree(tmp);
+  c->mem.release(tmp, b_tmp);
   if (ce != cudaSuccess) {
     oc->rp = nullptr;
     return cuda_fail(ce, "source order: landmarks");
@@ -108,7 +112,7 @@ bc_status build_cache(Graph *g, const DeviceGraph *dg, int T, cudaStream_t st, T
   if (L == 0) return BC_OK;
   int32_t *d_lm = nullptr, *d_depth = nullptr;
   const size_t b_lm = (size_t)L * 4, b_depth = (size_t)L * n * 4, b_out = (size_t)L * n;
-  bc_status s = c->mem.alloc((void **)&d_lm, b_lm);
+  s = c->mem.alloc((void **)&d_lm, b_lm);
   if (!s) s = c->mem.alloc((void **)&d_depth, b_depth);
   if (!s) s = c->mem.alloc((void **)&oc->d, b_out);
   if (!s && cudaMemcpyAsync(d_lm, lm.data(), b_lm, cudaMemcpyHostToDevice, st) != cudaSuccess)

@@ -113,6 +113,7 @@ struct TileSum {
   unsigned long long reached, reached_arcs;
 };
 constexpr int kTileBatch = 64;  // tiles launched before the host reads their sums
+constexpr size_t kBatchBytes = 16 + kTileBatch * sizeof(TileSum);  // stop word, then the sums
 
 }  // namespace
 
@@ -2584,7 +2585,7 @@ static bc_status ws_main(Ctx *ctx, TileWS *ws, int n, int T, cudaStream_t st) {
   const int G = T / 32;
   const size_t N = (size_t)n, NG = N * G, NT = N * T;
   const size_t bytes = NG * 4 * 5 + NT * 16 + (N / 32 + 1) * 4 + (N + 3) * 4 + (N + 3) * 8 + N * 24 +
-                       T * 8 + sizeof(TileCtl);
+                       T * 8 + sizeof(TileCtl) + kBatchBytes;
   bc_status s = ctx->mem.alloc(nullptr, bytes);
   if (s) return s;
   cudaError_t e = cudaSuccess;
@@ -2605,7 +2606,7 @@ static bc_status ws_main(Ctx *ctx, TileWS *ws, int n, int T, cudaStream_t st) {
   TA(ws->Fdone, N * 4);
   TA(ws->wsrc, (size_t)T * 8);
   TA(ws->ctl, sizeof(TileCtl));
-  TA(ws->stop, 16 + kTileBatch * sizeof(TileSum));
+  TA(ws->stop, kBatchBytes);
   ws->n = n;
   ws->T = T;
   ws->G = G;
