@@ -223,15 +223,30 @@ def code_sha1(path: str) -> str:
     return hashlib.sha1("\n".join(ln for ln in lines if ln.strip()).encode()).hexdigest()
 
 
+def kernel_sha1(name: str) -> str:
+    """sha1 over code_sha1 of a csrc file and of every file of this repository that it includes,
+    directly or through another (a change in a header's arithmetic changes the kernel too)."""
+    import hashlib
+    import re
+    todo, seen = [os.path.join(ROOT, "paper_1602_00963_gb300", "csrc", name)], []
+    while todo:
+        path = os.path.normpath(todo.pop(0))
+        if path in seen:
+            continue
+        seen.append(path)
+        with open(path) as f:
+            todo += [os.path.join(os.path.dirname(path), x) for x in re.findall(r'^\s*#include "([^"]+)"', f.read(), re.M)]
+    return hashlib.sha1("".join(code_sha1(p) for p in sorted(seen, key=os.path.basename)).encode()).hexdigest()
+
+
 def ncu_traffic(T: int, tiles_bytes: float):
     """DRAM bytes (read + write) per launch of the tile kernel from the committed ncu
     summary, if it was taken on the current kernel code and this tile width."""
     path = os.path.join(ROOT, "profiles", f"tile_rmat20_dram_T{T}.json")
-    src = os.path.join(ROOT, "paper_1602_00963_gb300", "csrc", "bc_tile.cu")
     try:
         with open(path) as f:
             j = json.load(f)
-        if j.get("kernel_code_sha1") != code_sha1(src) or int(j.get("tile_width", 0)) != T:
+        if j.get("kernel_code_sha1") != kernel_sha1("bc_tile.cu") or int(j.get("tile_width", 0)) != T:
             return None
         return float(j["dram_bytes_per_launch"])
     except (OSError, KeyError, ValueError):
