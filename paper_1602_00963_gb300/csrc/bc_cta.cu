@@ -1195,13 +1195,13 @@ static bc_status cta_plan(Ctx *ctx, int n, int max_degree, int units, bool tri, 
   return BC_OK;
 }
 
-static bc_status cta_alloc(Ctx *ctx, CtaWS **wsp, int n, int rows, size_t b_gws, bool row4) {
+static bc_status cta_alloc(Ctx *ctx, CtaWS **wsp, int n, int rows, size_t b_gws) {
   CtaWS *ws = new (std::nothrow) CtaWS();
   if (!ws) return fail(BC_ENOMEM, "host allocation failed");
   ws->n = n;
   ws->rows = rows;
   ws->b_gws = b_gws;
-  const size_t b_bcp = (size_t)rows * n * 8, b_row = row4 ? (size_t)n * 16 : 0;
+  const size_t b_bcp = (size_t)rows * n * 8;
   ws->bytes = b_bcp + b_gws + 64 + 2 * (kCtaMaxReq + 1) * sizeof(int32_t);
   bc_status s = ctx->mem.alloc(nullptr, ws->bytes);
   if (s) {
@@ -1217,19 +1217,24 @@ static bc_status cta_alloc(Ctx *ctx, CtaWS **wsp, int n, int rows, size_t b_gws,
     cta_free(ctx, ws);
     return fail(BC_ENOMEM, "CTA per-source workspace allocation failed");
   }
-  // row records where the budget leaves room (the kernel reads rp and ci without them)
-  if (b_row && (!ctx->mem.budget || ctx->mem.used.load() + 4 * b_row < ctx->mem.budget) &&
-      ctx->mem.alloc(nullptr, b_row) == BC_OK) {
-    if (cudaMalloc((void **)&ws->row4, b_row) == cudaSuccess) {
-      ws->bytes += b_row;
-    } else {
-      cudaGetLastError();
-      ws->row4 = nullptr;
-      ctx->mem.release(nullptr, b_row);
-    }
-  }
   *wsp = ws;
   return BC_OK;
+}
+
+// Row records where the budget leaves room (the kernel reads rp and ci without them), at the first call
+// whose state lies in global memory.
+static void cta_row_records(Ctx *ctx, CtaWS *ws, const CtaPlan &pl) {
+  const size_t b_row = (size_t)ws->n * 16;
+  if (pl.kind == 1 || ws->row4 || (ctx->mem.budget && ctx->mem.used.load() + 4 * b_row >= ctx->mem.budget) ||
+      ctx->mem.alloc(nullptr, b_row) != BC_OK)
+    return;
+  if (cudaMalloc((void **)&ws->row4, b_row) == cudaSuccess) {
+    ws->bytes += b_row;
+  } else {
+    cudaGetLastError();
+    ws->row4 = nullptr;
+    ctx->mem.release(nullptr, b_row);
+  }
 }
 
 // Bytes of a CTA's slice in a plan's layout (a second state and c's records only with triples).
@@ -1260,10 +1265,12 @@ static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, int64_t units, const C
     if (ncta < 1) return fail(BC_ENOMEM, "CTA per-source workspace exceeds the context HBM budget");
   }
   *max_cta = have;
-  if (have >= ncta) return BC_OK;
+  if (have >= ncta) {
+    cta_row_records(ctx, ws, pl);
+    return BC_OK;
+  }
   int rows = ncta;
   size_t b_gws = slice * ncta;
-  bool row4 = pl.kind != 1;
   if (same) {
     const int grown = std::max(ncta, (int)std::min<size_t>({(size_t)pl.ncta, (size_t)2 * have, room / per_cta}));
     const int r2 = std::max(grown, ws->rows);
@@ -1272,14 +1279,15 @@ static bc_status cta_ensure(Ctx *ctx, CtaWS **wsp, int n, int64_t units, const C
       rows = r2;
       b_gws = g2;
     }
-    row4 = row4 || ws->row4;
   }
   cta_free(ctx, ws);
   *wsp = nullptr;
-  bc_status s = cta_alloc(ctx, wsp, n, rows, b_gws, row4);
-  if (s && (rows != ncta || b_gws != slice * ncta)) s = cta_alloc(ctx, wsp, n, ncta, slice * ncta, row4);
-  if (!s) *max_cta = (int)std::min<size_t>({(size_t)(*wsp)->rows, (*wsp)->b_gws / slice, (size_t)pl.ncta});
-  return s;
+  bc_status s = cta_alloc(ctx, wsp, n, rows, b_gws);
+  if (s && (rows != ncta || b_gws != slice * ncta)) s = cta_alloc(ctx, wsp, n, ncta, slice * ncta);
+  if (s) return s;
+  *max_cta = (int)std::min<size_t>({(size_t)(*wsp)->rows, (*wsp)->b_gws / slice, (size_t)pl.ncta});
+  cta_row_records(ctx, *wsp, pl);
+  return BC_OK;
 }
 
 bool cta_fits(int32_t n) { return n > 0 && n <= kCtaMaxN; }

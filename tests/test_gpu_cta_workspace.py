@@ -64,3 +64,17 @@ def test_layouts_taking_turns(ctx):
     assert_bc_close(b, want, what="single sources")
     assert changes(free[1:]) == 0  # after one call of each the workspace serves both
     bc.bc_destroy(h)
+
+
+def test_row_records_after_a_shared_layout(ctx):
+    """A call with its state in global memory builds its row records (one launch more) whatever
+    workspace an earlier call of another layout left."""
+    g = gg.subdivide_edges(gg.ba_pref_attach(1500, 3), 0.1, 5)
+    launches = []
+    for before in (None, CTA):
+        h = upload(ctx, g)
+        if before is not None:
+            bc.bc_exact(h, g.n, before)
+        launches.append(bc.bc_exact(h, g.n, bc.BC_DEG2)[1]["kernel_launches"])
+        bc.bc_destroy(h)
+    assert launches == [launches[0]] * 2 and launches[0] >= 3
