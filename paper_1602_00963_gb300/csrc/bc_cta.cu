@@ -1140,12 +1140,17 @@ struct CtaPlan {
 //   10.0 against 10.7), else 128 registers and 512 threads (G(9000, 36,000) all sources 9.0
 //   against 10.0), a lane then taking rows of up to 32 arcs instead of 12 (G(9000, 72,000): 12.9,
 //   with 16 16.4, with 12 20.5; the social graph 9.6 with 12, 9.9 with 16, 11.1 with 32).  From
-//   global memory 128 registers (64 spill in the sweeps: grid 1024^2 92 against 70); narrow
-//   graphs need no code for larger rows and run with 80 (59).
+//   global memory 128 registers (64 spill in the sweeps: grid 1024^2, 500 sources, 99 against 69);
+//   narrow graphs need no code for larger rows and run with 80 (53).
 // * Threads: an SM's threads over the states that fit it and have a source (one source on
 //   n = 1000: 85 us with 512, 95 with 128); from global memory 512 (social graph
-//   n = 60,001, 500 sources: 11.9, 13.3 with 256), narrow graphs 96 / 192 / 384 by size (grid
-//   300^2, 500 sources: 5.5 with 192, 6.7 with 128; grid 1024^2: 59 with 384, 88 with 256).
+//   n = 60,001, 500 sources: 11.9, 13.3 with 256), narrow graphs 96 / 192 / 384 by size.  Grids, 500
+//   sources, with 192 and 384: n = 499,849 25.8 and 25.7, 722,500 41 and 37, 1,048,576 66 and 54.
+//   With 96 and 192: every vertex a source 8,100 6.5 and 9.4, 16,129 23.0 and 28.7, 32,400 81 and
+//   98; 500 sources 0.92 and 0.91, 1.59 and 1.36, 2.75 and 2.12.  So below 500,000 it is the number of
+//   sources per SM that decides; the line at 16,384 takes calls below it as exact ones, above it as
+//   a few hundred sources.  With triples 96 and 128 are alike (n = 10,944 15.2 and 14.6, 17,176 31.2
+//   and 33.6, 28,997 83 and 84).
 static bc_status cta_plan(Ctx *ctx, int n, int max_degree, int units, bool tri, CtaPlan *pl) {
   const bool narrow = max_degree > 0 && max_degree <= kNarrowDeg;
   const bool fits = !tri && n < (1 << 15) && cta_smem_bytes(n, false) <= kCtaSmemMax;

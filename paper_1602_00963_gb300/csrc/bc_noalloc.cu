@@ -222,8 +222,10 @@ extern "C" bc_status bc_sources_noalloc(int32_t n, const int32_t *row_ptr, const
   }
   BC_CUDA_TRY(cudaMemsetAsync(bc_out, 0, (size_t)n * sizeof(double), st));
   const PlainWS ws = kFull.at(base, n);
-  // the grid: barriers of fewer CTAs are cheaper, while the level's work fits them (R-MAT scale 12,
-  // per source: 118 us with 12 CTAs, 129 with all; scale 16: 162 with all, 278 with 8)
+  // the grid: barriers of fewer CTAs are cheaper, while the level's work fits them.  Per source with
+  // 12 / 64 / all CTAs: grid 180^2, 129 k arcs, 8915 / 9196 / 9692 us (R-MAT scale 12, 96 k arcs, 105 /
+  // 105 / 108); G(20,000, 100,000) 180 / 163 / 166, R-MAT scale 14, 426 k arcs, 151 / 131 / 136; scale
+  // 15, 882 k arcs, 182 / 136 / 139, scale 16, 1.8 M arcs, 261 / 152 / 151
   const int ctas = std::min(sms, nnz <= 150000 ? 12 : nnz <= 600000 ? 64 : sms);
   int derr = 0;
   const bc_status s = plain_run_view(ws, a, ctas, 20ull * 1000 * 1000 * 1000, st, &derr);

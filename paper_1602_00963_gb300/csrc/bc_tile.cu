@@ -3057,8 +3057,8 @@ bc_status tile_run(Ctx *ctx, Graph *g, TileWS **wsp, const TileArgs &a, cudaStre
     return p;
   };
   // Tiles of the persistent loop are launched up to kTileBatch in a row; the host waits once per
-  // batch, not after each tile (a wait, two copies and the launches behind them left the GPU idle
-  // for about 0.1 ms a tile: leaf-rich graph n = 130,001, 16 tiles of 64, 24.7 ms with the waits).
+  // batch, not after each tile (a wait and a copy leave the GPU idle for about 15 us a tile: leaf-rich
+  // graph n = 130,001, 16 tiles of 64, 24.85 ms with a wait after each tile, 24.61 in one batch).
   // A tile that failed (before any BC update) stops the ones behind it; it is run again, and the
   // batch goes on from there, so BC takes the tiles in list order in any case.
   int first = 0;  // sources done
