@@ -575,9 +575,9 @@ __device__ __forceinline__ int cta_forward(const CtaK &p, const CtaState<SM> &S,
             allx = allx && (r[j].tag & 1u);
           }
         }
-        // u < dl: this row's own step.  The loop goes on for longer rows of the warp, and a step
+        // u == 0: the one step of such a row.  The loop goes on for longer rows of the warp, and a step
         // without parents would leave the sum with the exponent of none.
-        if (!SM && u < dl && ov && !xp && row.deg <= kThin) {
+        if (!SM && u == 0 && ov && !xp && row.deg <= kThin) {
           if (allx) {  // mantissas brought to the largest exponent (exact) and added in arc order
             a.e = INT_MIN;
 #pragma unroll
